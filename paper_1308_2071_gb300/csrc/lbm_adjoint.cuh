@@ -9,7 +9,7 @@
 // checked against finite differences of the forward functions.
 #pragma once
 
-#include "lbm_device.cuh"
+#include "lbm_node.cuh"
 
 namespace lbm {
 

@@ -178,6 +178,71 @@ void fill_coef(const lbm_params* p, const Derived& dv, Coef<R>* c) {
     c->fq = (R)fq;
     c->ifq = (R)(1.0 / fq);
     c->wt1fq = (R)((4.0 + p->varpi) / 20.0) * (R)fq;
+
+    // the constants of lbm_core.cuh (see there for the rearranged formulas),
+    // formed in FP64; with a porosity field 1 / phi comes with the products
+    Coll<R>& k = c->k;
+    const bool field = p->use_phi_field != 0;
+    const double ip = field ? 1.0 : 1.0 / p->phi;
+    const double hs[9] = {1 - s[0] / 2, 1 - s[1] / 2, 1 - s[2] / 2, 1 - s[3] / 2, 1 - s[4] / 2,
+                          1 - s[5] / 2, 1 - s[6] / 2, 1 - s[7] / 2, 1 - s[8] / 2};
+    const double c_lin = p->phi * dv.nu / dv.K, c_quad = p->phi * dv.Fphi / sqrt(dv.K);
+    k.hb = (R)(0.5 * dv.gbeta * (field ? 1.0 : p->phi));
+    k.gb = (R)dv.gbeta;
+    k.cc = (R)(0.25 * (field ? (double)c->a_lin : c_lin));
+    k.ec = field ? (R)0 : (R)(0.25 * c_lin + 0.0625 * c_lin * c_lin);
+    k.l1 = (R)(0.5 * (field ? (double)c->a_quad : c_quad));
+    k.iphi = (R)(1.0 / p->phi);
+    k.niphi = (R)(-1.0 / p->phi);
+    k.qhalf = c->qhalf;
+    k.a0 = (R)(-(s[0] + 4 * s[1] + 4 * s[2]) / 9);
+    k.b0 = (R)((-s[0] - s[1] + 2 * s[2]) / 9);
+    k.c0 = (R)((-s[0] + 2 * s[1] - s[2]) / 9);
+    k.a1 = (R)((s[1] - s[2]) / 15);
+    k.b1 = (R)((s[1] + 2 * s[2]) / 60);
+    k.c1 = (R)(-(2 * s[1] + s[2]) / 60);
+    k.a2 = (R)(-(hs[1] + hs[2]) * 12 / 9 * ip);
+    k.b2 = (R)((2 * hs[2] - hs[1]) / 3 * ip);
+    k.c2 = (R)((2 * hs[1] - hs[2]) / 3 * ip);
+    k.k7 = (R)(-s[7] / 4);
+    k.f7 = (R)(hs[7] * ip);
+    k.k8 = (R)(-s[8] / 4);
+    k.f8 = (R)(hs[8] / 2 * ip);
+    k.s4d = (R)(-s[4] / 12);  // the axis part is exactly -2 times the diagonal one
+    k.s4a = (R)-2 * k.s4d;
+    k.s6d = (R)(-s[6] / 12);
+    k.s6a = (R)-2 * k.s6d;
+    k.s3 = (R)(s[3] / 6);
+    k.s4 = (R)(s[4] / 6);
+    k.s5 = (R)(s[5] / 6);
+    k.s6 = (R)(s[6] / 6);
+    k.f5 = (R)(hs[5] / 6);
+    k.f6 = (R)(hs[6] / 6);
+    k.is = c->inv_sigma;
+    k.Tis = (R)(dv.T0 / p->sigma);
+    k.nis = -k.is;
+    k.nTis = -k.Tis;
+    const double psi = dv.Q / p->sigma, wt0 = (1.0 - p->varpi) / 5.0, wt1 = (4.0 + p->varpi) / 20.0;
+    k.q0 = (R)(wt0 * psi);
+    k.q1 = (R)(wt1 * psi);
+    k.t1 = (R)(-z[3] / 20 * (1.0 - p->varpi));
+    k.h1 = (R)(z[3] / 20 * (4.0 + p->varpi));
+    k.t4 = (R)-4 * k.t1;
+    k.h4 = (R)-4 * k.h1;
+    k.z1 = (R)(-z[1] / 2);
+    k.z2 = (R)(-z[2] / 2);
+    k.z4 = (R)(-z[4] / 4);
+    k.nz4 = -k.z4;
+    const double fu = p->precision == LBM_F32 || p->precision == LBM_F32_STORE_F16 ? fq : 1.0;
+    k.fu = (R)fu;
+    k.ifu = (R)(1.0 / fu);
+    k.w1 = (R)wt1 * (R)fu;
+    k.nw0 = -(R)wt0 * (R)fu;
+    k.nw1 = -k.w1;
+    k.wt0 = (R)wt0;
+    k.wt1 = (R)wt1;
+    k.dTh = c->dTh;
+    k.dTc = c->dTc;
 }
 
 }  // namespace

@@ -73,6 +73,22 @@ __host__ __device__ __forceinline__ Coef<R> with_cavity_rates(const Coef<R>& cu,
     c.c_quad = v.c_quad;
     c.a_lin = v.a_lin;
     c.a_quad = v.a_quad;
+    c.k.hb = v.k.hb;
+    c.k.gb = v.k.gb;
+    c.k.cc = v.k.cc;
+    c.k.ec = v.k.ec;
+    c.k.l1 = v.k.l1;
+    c.k.iphi = v.k.iphi;
+    c.k.niphi = v.k.niphi;
+    c.k.a2 = v.k.a2;
+    c.k.b2 = v.k.b2;
+    c.k.c2 = v.k.c2;
+    c.k.k7 = v.k.k7;
+    c.k.f7 = v.k.f7;
+    c.k.k8 = v.k.k8;
+    c.k.f8 = v.k.f8;
+    c.k.z1 = v.k.z1;
+    c.k.z2 = v.k.z2;
     return c;
 }
 

@@ -10,7 +10,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/lbm.h"
-#include "lbm_device.cuh"
+#include "lbm_node.cuh"
 
 namespace lbm {
 

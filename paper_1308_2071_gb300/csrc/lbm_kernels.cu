@@ -34,17 +34,24 @@ __global__ void __launch_bounds__(256) k_step(Src<T> src, Dst<T> dst, const type
     update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x, y, status, obs);
 }
 
+// Blocks of 256 threads per SM that the two-node kernels are compiled for (see k_step2).
+template <class T> constexpr int step_blocks() {
+    return sizeof(typename T::R) == 8 ? 1 : sizeof(typename T::SF) == 4 ? 3 : 4;
+}
+
 // Two nodes per thread, (x, y) and (x, y + blockDim.y): when both are fluid
 // nodes all 28 loads are issued before any arithmetic, doubling the bytes in
 // flight per thread (the FP16-flow variant moves 38 B per node, too few to
 // cover HBM latency with one node per thread).  Wall nodes take the general
 // path one at a time.
-// FP32 arithmetic: at most 64 registers (4 blocks of 256 threads, 8 of 128
-// per SM), which measured faster than the unconstrained 68-80 registers at
-// every size and storage type: more warps keep more loads in flight.  FP64
-// would spill under that limit.
+// FP32 storage: at most 80 registers (3 blocks of 256 threads, 6 of 128 per
+// SM), where the paired collision spills nothing (140 bytes under 64).  Measured
+// at 4096^2 / 1024^2 / 512^2 / 200^2: 273.7 / 17.7 / 5.5 / 3.1 us per step, under
+// 64 registers 310.7 / 22.8 / 7.3 / 3.7, with the collision before this form 274.7 /
+// 20.1 / 7.2 / 4.4.  FP16 flow: at most 64 (4 blocks), which its direct form fits.
+// FP64 would spill under either limit.
 template <class T, bool FIELD, bool OBS>
-__global__ void __launch_bounds__(256, sizeof(typename T::R) == 4 ? 4 : 1)
+__global__ void __launch_bounds__(256, step_blocks<T>())
     k_step2(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
             int* __restrict__ status, double* __restrict__ obs) {
     wait_for_previous_step();
@@ -60,7 +67,7 @@ __global__ void __launch_bounds__(256, sizeof(typename T::R) == 4 ? 4 : 1)
 // aligned pairs (8-byte FP32, 4-byte FP16 accesses), a third fewer memory
 // instructions than two nodes apart along y.  Same register cap.
 template <class T, bool FIELD, bool OBS>
-__global__ void __launch_bounds__(256, sizeof(typename T::R) == 4 ? 4 : 1)
+__global__ void __launch_bounds__(256, step_blocks<T>())
     k_step2x(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
              int* __restrict__ status, double* __restrict__ obs) {
     wait_for_previous_step();
