@@ -17,7 +17,7 @@ using namespace lbm;
 
 namespace {
 
-constexpr int kGraphSteps = 64;  // steps per captured graph (even: keeps buffer parity)
+constexpr int kGraphSteps = 64;  // steps per captured graph (an even number of launches: keeps buffer parity)
 
 thread_local std::string g_init_error;
 
@@ -54,6 +54,7 @@ struct lbm_handle_s {
     double* steady_dev = nullptr;       // 8 doubles of loop state
     double* extrema_dev = nullptr;      // 3 doubles per column
     int bx = 128, by = 2, npt = 1;
+    DuoShape duo;       // two steps per launch (threads = 0: not on this lattice)
     std::string err;
 };
 
@@ -336,15 +337,54 @@ StepLaunch step_launch(lbm_handle h, int src, cudaStream_t s) {
     return L;
 }
 
-// nsteps steps from buf[cur] in the handle's launch shape, the first launched
-// as a programmatic dependent when pdl_first (a step kernel right before it).
-int advance(lbm_handle h, long nsteps, bool pdl_first) {
-    for (long k = 0; k < nsteps; ++k) {
-        StepLaunch Ls = step_launch(h, h->cur, h->stream);
-        Ls.pdl = k > 0 || pdl_first;
-        CK(h, launch_step(Ls, h->coef));
-        h->cur ^= 1;
+// The most steps that one launch takes on this lattice where the state between
+// is not needed: two (lbm_duo.cu) or one.
+int most_steps(lbm_handle h) { return h->duo.threads ? 2 : 1; }
+
+// Two steps per launch for FP32 storage (FP64 is bound by its arithmetic unit,
+// and the states between of FP16 flow have to be rounded) from 2^18 nodes on.
+// Measured, us per step with one step per launch / two: 384^2 4.2 / 5.1, 601 x
+// 397 4.8 / 5.4, 512^2 5.3 / 5.3, 1024^2 17.8 / 14.0, 4096^2 274 / 170.
+cudaError_t choose_steps(lbm_handle h) {
+    constexpr long kTwosWorth = 1 << 18;  // nodes
+    if ((long)h->p.nx * h->p.ny < kTwosWorth) return cudaSuccess;
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    return duo_shape(h->precision, h->p.use_phi_field != 0, h->gm, nsm, &h->duo);
+}
+
+cudaError_t launch_steps(lbm_handle h, const StepLaunch& Ls, int steps) {
+    return steps == 1 ? launch_step(Ls, h->coef) : launch_duo(Ls, h->coef, h->duo);
+}
+
+// nsteps steps from buf[cur] on stream s, several per launch where possible;
+// the first is launched as a programmatic dependent when pdl_first (a step
+// kernel right before it), the others when pdl.  keep_prev: the last step is
+// one of its own, so that buf[cur ^ 1] ends up holding B_{n-1}, from which the
+// post-stream state is rebuilt.  even: in an even number of launches, which
+// leaves cur as it was (nsteps even).
+cudaError_t enqueue_steps(lbm_handle h, long nsteps, cudaStream_t s, bool pdl_first, bool pdl, bool keep_prev,
+                          bool even) {
+    if (nsteps <= 0) return cudaSuccess;
+    const long alone = keep_prev ? 1 : 0, together = nsteps - alone;
+    long launches = (together + most_steps(h) - 1) / most_steps(h);
+    if (even && ((launches + alone) & 1)) ++launches;
+    cudaError_t e = cudaSuccess;
+    for (long k = 0; k < launches + alone && e == cudaSuccess; ++k) {
+        // the steps taken together, shared out evenly
+        const int steps = k < launches ? (int)(together * (k + 1) / launches - together * k / launches) : 1;
+        StepLaunch Ls = step_launch(h, h->cur, s);
+        Ls.pdl = k == 0 ? pdl_first : pdl;
+        if ((e = launch_steps(h, Ls, steps)) == cudaSuccess) h->cur ^= 1;
     }
+    return e;
+}
+
+// The same on the handle's stream, in the handle's launch shape.
+int advance(lbm_handle h, long nsteps, bool pdl_first, bool keep_prev) {
+    CK(h, enqueue_steps(h, nsteps, h->stream, pdl_first, true, keep_prev, false));
     return LBM_OK;
 }
 
@@ -366,12 +406,10 @@ int reset_state(lbm_handle h) {
 int capture_graph(lbm_handle h, int parity) {
     cudaGraph_t g = nullptr;
     CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int src = parity;
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < kGraphSteps && e == cudaSuccess; ++k) {
-        e = launch_step(step_launch(h, src, h->cap_stream), h->coef);
-        src ^= 1;
-    }
+    const int cur = h->cur;
+    h->cur = parity;
+    cudaError_t e = enqueue_steps(h, kGraphSteps, h->cap_stream, false, true, false, true);
+    h->cur = cur;
     cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
     if (e != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -415,11 +453,10 @@ int build_steady_graph(lbm_handle h, long K, long max_checks, double tol) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(h->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            int src = h->cur;
-            for (long k = 0; k < K && e == cudaSuccess; ++k) {
-                e = launch_step(step_launch(h, src, h->cap_stream), h->coef);
-                src ^= 1;
-            }
+            // an even number of launches: every turn of the loop starts from the same buffer
+            const int cur = h->cur;
+            e = enqueue_steps(h, K, h->cap_stream, false, true, true, true);
+            h->cur = cur;
             if (e == cudaSuccess) {
                 SteadyCheckLaunch L;
                 L.precision = h->precision;
@@ -512,6 +549,7 @@ int lbm_init(const lbm_params* p, void* stream, lbm_handle* out) {
             return fail(nullptr, LBM_ERR_CUDA, m_);                 \
         }                                                           \
     } while (0)
+    CKI(choose_steps(h));
     CKI(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     CKI(cudaMalloc(&h->buf[0], h->buf_bytes));
     CKI(cudaMalloc(&h->buf[1], h->buf_bytes));
@@ -650,7 +688,14 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
             h->bx = cd[0];
             h->by = cd[1];
             h->npt = cd[2];
-            int rc = advance(h, 3, false);
+            auto singles = [&](long n) {
+                for (long k = 0; k < n; ++k) {
+                    int r1 = advance(h, 1, k > 0, true);
+                    if (r1 != LBM_OK) return r1;
+                }
+                return (int)LBM_OK;
+            };
+            int rc = singles(3);
             if (rc != LBM_OK) return rc;
             // 30 steps, or on small lattices as many as take about 2 ms (at most
             // 2000), so that timer resolution and clock ramps do not pick the shape
@@ -658,7 +703,7 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
             float ms = 0.f;
             for (int pass = 0; pass < 2; ++pass) {
                 CK(h, cudaEventRecord(e0, h->stream));
-                if ((rc = advance(h, nsteps, false)) != LBM_OK) return rc;
+                if ((rc = singles(nsteps)) != LBM_OK) return rc;
                 CK(h, cudaEventRecord(e1, h->stream));
                 CK(h, cudaEventSynchronize(e1));
                 CK(h, cudaEventElapsedTime(&ms, e0, e1));
@@ -700,20 +745,18 @@ int lbm_step(lbm_handle h, long nsteps) {
     if (!h) return fail(nullptr, LBM_ERR_ARG, "handle is NULL");
     if (nsteps < 0) return fail(h, LBM_ERR_ARG, "nsteps < 0");
     long left = nsteps;
-    while (left >= kGraphSteps) {
+    // with several steps per launch the graphs leave no B_{n-1}: at least one step follows them
+    const long after = most_steps(h) > 1 ? 1 : 0;
+    while (left >= kGraphSteps + after) {
         if (!h->gexec[h->cur]) {
             int rc = capture_graph(h, h->cur);
             if (rc != LBM_OK) return rc;
         }
         CK(h, cudaGraphLaunch(h->gexec[h->cur], h->stream));
-        left -= kGraphSteps;  // even count: cur unchanged
+        left -= kGraphSteps;  // an even number of launches: cur unchanged
     }
-    for (long k = 0; left > 0; --left, ++k) {
-        StepLaunch Ls = step_launch(h, h->cur, h->stream);
-        Ls.pdl = k > 0;  // directly behind the previous step kernel
-        CK(h, launch_step(Ls, h->coef));
-        h->cur ^= 1;
-    }
+    int rc = advance(h, left, false, true);  // each directly behind the step kernel before it
+    if (rc != LBM_OK) return rc;
     h->t += nsteps;
     return LBM_OK;
 }
@@ -942,7 +985,8 @@ int lbm_adjoint_step(lbm_handle h, long nsteps, long ckpt_every, double* J, void
             }
             const long next = (j / K + 1) * K - 1;  // the next step that keeps its input state
             const long upto = next <= N - 2 ? next : N;
-            rc = advance(h, upto - t, t > 0 && !copy);  // directly behind the previous step kernel
+            // directly behind the previous step kernel; only the last run's B_{N-1} is read
+            rc = advance(h, upto - t, t > 0 && !copy, upto == N);
             t = upto;
         }
         h->t = N;

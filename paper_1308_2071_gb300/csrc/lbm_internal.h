@@ -109,6 +109,14 @@ struct ReadStateLaunch {
 };
 
 cudaError_t launch_step(const StepLaunch& L, const CoefSet& cs);
+// Two steps at once (lbm_duo.cu): dst receives B_{n+2} from src = B_n, with the
+// bits of two launch_step calls.  Strips of `width` node pairs and segments of
+// `rows` rows on blocks of `threads` threads; threads = 0: not on this lattice.
+struct DuoShape {
+    int threads = 0, width = 0, rows = 0, strips = 0, segs = 0;
+};
+cudaError_t duo_shape(int precision, bool field, const Geom& gm, int nsm, DuoShape* out);
+cudaError_t launch_duo(const StepLaunch& L, const CoefSet& cs, const DuoShape& s);
 cudaError_t launch_observe(const ObserveLaunch& L, const CoefSet& cs);
 cudaError_t launch_nusselt(const ObserveLaunch& L, const CoefSet& cs);
 cudaError_t launch_read_state(const ReadStateLaunch& L, const CoefSet& cs);

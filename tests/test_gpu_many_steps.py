@@ -1,0 +1,111 @@
+"""Several steps per launch: lbm_step(n) runs all but its last step in launches
+of several (tiles on chip on small lattices, two steps per launch on large
+ones) and must leave the lattice that n calls of lbm_step(1) leave, bit for
+bit, padding and frames included (every kernel runs the same explicit
+operations per node).  Sizes at the edges of the tiles, strips and segments
+(odd widths, whose right wall is alone in its pair of nodes; a strip or a
+segment more or less), every wall variant."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SMALL = [(5, 5), (6, 11), (8, 8), (9, 8), (17, 13), (64, 64), (65, 33), (66, 9), (129, 41), (190, 12), (257, 70), (7, 900)]
+# two steps per launch from 2^18 nodes: strips of up to 94 pairs, segments of up to 32 rows, wall tiles of 28 and 22 nodes
+LARGE = [(512, 512), (513, 511), (600, 437), (1021, 257), (1023, 259), (8, 32768), (9, 29500), (32771, 8), (26300, 10),
+         (1501, 1500)]
+SIZES = SMALL + LARGE
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def _pair(nx, ny, **kw):
+    from paper_1308_2071_gb300 import Cavity
+
+    base = dict(Ra=1e4, Da=1e-2, phi=0.6, precision="f32")
+    base.update(kw)
+    return Cavity(nx, ny, **base), Cavity(nx, ny, **base)
+
+
+def _same(a, b, n):
+    for _ in range(n):
+        a.step(1)
+    b.step(n)
+    assert a.query() == b.query()
+    assert bytes(a.save()) == bytes(b.save())
+    # and the lattice after it, from the other buffer
+    a.step(1)
+    b.step(1)
+    assert bytes(a.save()) == bytes(b.save())
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("precision", ["f32", "f32t"])
+def test_steps_in_twos_leave_the_same_bits(size, precision):
+    a, b = _pair(*size, precision=precision)
+    _same(a, b, 13)
+
+
+@pytest.mark.parametrize("size", [(70, 50), (640, 420)])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 7, 64, 65, 66, 131])
+def test_every_count_of_steps(size, n):
+    a, b = _pair(*size)
+    _same(a, b, n)
+
+
+@pytest.mark.parametrize("size", [(70, 50), (640, 420)])
+def test_the_steady_loop_takes_the_same_steps(size):
+    # the loop's body runs its steps in an even number of launches, the last alone
+    for every in (2, 4, 6, 20, 33):
+        a, b = _pair(*size)
+        n, _ = b.run_steady(tol=1e-30, check_every=every, max_steps=3 * every)
+        assert n == 3 * (every + every % 2)
+        _same_state = a.step(n).save()
+        assert bytes(_same_state) == bytes(b.save()) and a.query() == b.query()
+        a.close()
+        b.close()
+
+
+@pytest.mark.parametrize("size", [(9, 8), (64, 64), (129, 41), (700, 395), (701, 394)])
+@pytest.mark.parametrize("kw", [dict(thermal_bc=1, Ra=0.0, phi=1.0, Pr=7.0, RaI=6.4e4, forchheimer=0),
+                                dict(RaI=1e5, Pr=0.7, Th=1.5, Tc=-0.25), dict(Da=float("inf"), forchheimer=0),
+                                dict(collision=1), dict(adiabatic_order=2), "field"])
+def test_wall_and_parameter_variants(size, kw):
+    import torch
+
+    from paper_1308_2071_gb300.inputs import perturbed_porosity
+
+    if kw == "field":
+        phi = perturbed_porosity(size[1], size[0], phi_bar=0.6, amplitude=0.1, corr_len=6.0, seed=3)
+        kw = dict(phi_field=torch.from_numpy(phi).cuda())
+    a, b = _pair(*size, **kw)
+    _same(a, b, 12)
+
+
+@pytest.mark.parametrize("size", [(70, 50), (640, 420)])
+def test_divergence_between_two_steps_of_a_launch_is_flagged(size):
+    # a NaN planted in the lattice spreads and raises the flag, also when the
+    # first step that meets it is one whose lattice stays on chip
+    from paper_1308_2071_gb300 import Cavity, _lib
+
+    nx, ny = size
+    pitch = -(-nx // 32) * 32
+    c = Cavity(nx, ny, Ra=1e4, Da=1e-2, phi=0.6, precision="f32")
+    c.step(5)
+    blob = c.save()
+    arr = np.frombuffer(blob, dtype=np.float32, count=14 * pitch * ny, offset=40)
+    arr.setflags(write=True)
+    arr[1 * pitch * ny + 25 * pitch + 33] = np.nan
+    c.load(blob)
+    c.step(9)
+    assert c.query()[1] == _lib.LBM_ERR_DIVERGED
+    c.close()
