@@ -54,6 +54,7 @@ struct lbm_handle_s {
     double* steady_dev = nullptr;       // 8 doubles of loop state
     double* extrema_dev = nullptr;      // 3 doubles per column
     int bx = 128, by = 2, npt = 1;
+    TileShape tile;     // several steps per launch on chip (steps = 0: not on this lattice)
     DuoShape duo;       // two steps per launch (threads = 0: not on this lattice)
     std::string err;
 };
@@ -337,26 +338,40 @@ StepLaunch step_launch(lbm_handle h, int src, cudaStream_t s) {
     return L;
 }
 
-// The most steps that one launch takes on this lattice where the state between
-// is not needed: two (lbm_duo.cu) or one.
-int most_steps(lbm_handle h) { return h->duo.threads ? 2 : 1; }
+// The most steps that one launch takes on this lattice where the states
+// between are not needed: tiles on chip (lbm_tile.cu), two steps per launch
+// (lbm_duo.cu), or one.
+int most_steps(lbm_handle h) { return h->tile.steps ? h->tile.steps : h->duo.threads ? 2 : 1; }
 
-// Two steps per launch for FP32 storage (FP64 is bound by its arithmetic unit,
-// and the states between of FP16 flow have to be rounded) from 2^18 nodes on.
-// Measured, us per step with one step per launch / two: 384^2 4.2 / 5.1, 601 x
-// 397 4.8 / 5.4, 512^2 5.3 / 5.3, 1024^2 17.8 / 14.0, 4096^2 274 / 170.
+// Picks the way (FP32 storage only: FP64 is bound by its arithmetic unit, and
+// the states between of FP16 flow have to be rounded).  Measured, us per step
+// with one step per launch / two / a tile on chip: 64^2 2.9 / 3.5 / 1.0, 200^2 3.0 /
+// 3.6 / 1.7, 384^2 4.2 / 5.1 / 3.3, 450^2 4.8 / 5.1 / 4.1, 601 x 397 4.8 / 5.4 / 5.0,
+// 512^2 5.3 / 5.3 / 5.9, 1024^2 17.8 / 14.0 / -, 4096^2 274 / 170 / -.
 cudaError_t choose_steps(lbm_handle h) {
+    constexpr double kTileWorth = 4.2;    // us per step of tile_shape's model (450^2: 3.8, 601 x 397: 4.3)
     constexpr long kTwosWorth = 1 << 18;  // nodes
-    if ((long)h->p.nx * h->p.ny < kTwosWorth) return cudaSuccess;
+    if (h->precision != PREC_F32 && h->precision != PREC_F32T) return cudaSuccess;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    return duo_shape(h->precision, h->p.use_phi_field != 0, h->gm, nsm, &h->duo);
+    const bool field = h->p.use_phi_field != 0;
+    const TileShape tile = tile_shape(h->p.nx, h->p.ny, nsm);
+    if (tile.steps && tile.us < kTileWorth) {
+        h->tile = tile;
+        return tile_prepare(h->precision, field);
+    }
+    if ((long)h->p.nx * h->p.ny >= kTwosWorth) return duo_shape(h->precision, field, h->gm, nsm, &h->duo);
+    return cudaSuccess;
 }
 
 cudaError_t launch_steps(lbm_handle h, const StepLaunch& Ls, int steps) {
-    return steps == 1 ? launch_step(Ls, h->coef) : launch_duo(Ls, h->coef, h->duo);
+    if (steps == 1) return launch_step(Ls, h->coef);
+    if (!h->tile.steps) return launch_duo(Ls, h->coef, h->duo);
+    TileShape s = h->tile;
+    s.steps = steps;
+    return launch_tile(Ls, h->coef, s);
 }
 
 // nsteps steps from buf[cur] on stream s, several per launch where possible;

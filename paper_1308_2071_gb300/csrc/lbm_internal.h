@@ -117,6 +117,16 @@ struct DuoShape {
 };
 cudaError_t duo_shape(int precision, bool field, const Geom& gm, int nsm, DuoShape* out);
 cudaError_t launch_duo(const StepLaunch& L, const CoefSet& cs, const DuoShape& s);
+// Several steps at once on a lattice that fits on chip (lbm_tile.cu): tx x ty
+// tiles, `steps` steps per launch (0, or at least 2), at about us microseconds
+// per step.  tile_prepare: once per device, before launch_tile.
+struct TileShape {
+    int tx = 0, ty = 0, steps = 0;
+    double us = 1e300;
+};
+TileShape tile_shape(int nx, int ny, int nsm);
+cudaError_t tile_prepare(int precision, bool field);
+cudaError_t launch_tile(const StepLaunch& L, const CoefSet& cs, const TileShape& s);
 cudaError_t launch_observe(const ObserveLaunch& L, const CoefSet& cs);
 cudaError_t launch_nusselt(const ObserveLaunch& L, const CoefSet& cs);
 cudaError_t launch_read_state(const ReadStateLaunch& L, const CoefSet& cs);
