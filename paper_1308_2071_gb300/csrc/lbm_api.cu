@@ -345,12 +345,12 @@ int most_steps(lbm_handle h) { return h->tile.steps ? h->tile.steps : h->duo.thr
 
 // Picks the way (FP32 storage only: FP64 is bound by its arithmetic unit, and
 // the states between of FP16 flow have to be rounded).  Measured, us per step
-// with one step per launch / two / a tile on chip: 64^2 2.9 / 3.5 / 1.0, 200^2 3.0 /
-// 3.6 / 1.7, 384^2 4.2 / 5.1 / 3.3, 450^2 4.8 / 5.1 / 4.1, 601 x 397 4.8 / 5.4 / 5.0,
-// 512^2 5.3 / 5.3 / 5.9, 1024^2 17.8 / 14.0 / -, 4096^2 274 / 170 / -.
+// with one step per launch / two / a tile on chip: 64^2 2.2 / 3.5 / 1.0, 200^2 2.3 /
+// 3.6 / 1.7, 384^2 3.4 / 5.1 / 3.3, 450^2 3.6 / 5.1 / 4.1, 601 x 397 4.3 / 5.4 / 5.0,
+// 700^2 6.3 / 7.2 / -, 850^2 9.3 / 9.3 / -, 1024^2 16.6 / 13.9 / -, 4096^2 272 / 170 / -.
 cudaError_t choose_steps(lbm_handle h) {
-    constexpr double kTileWorth = 4.2;    // us per step of tile_shape's model (450^2: 3.8, 601 x 397: 4.3)
-    constexpr long kTwosWorth = 1 << 18;  // nodes
+    constexpr double kTileWorth = 3.2;  // us per step of tile_shape's model (384^2: 3.0, 450^2: 3.8)
+    constexpr long kTwosWorth = 850000;  // nodes
     if (h->precision != PREC_F32 && h->precision != PREC_F32T) return cudaSuccess;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -541,12 +541,18 @@ int lbm_init(const lbm_params* p, void* stream, lbm_handle* out) {
     h->p = *p;
     h->precision = p->precision;
     const long plane = h->gm.plane;
-    // defaults (the autotuner's picks on the 4096^2 benchmark lattice): FP32
-    // arithmetic two nodes side by side along x in 128-thread blocks, FP64 two
-    // nodes along y
-    h->bx = p->block_x > 0 ? p->block_x : (p->nx <= 128 ? 32 : 64);
-    h->by = p->block_y > 0 ? p->block_y : (h->bx >= 128 ? 1 : 128 / h->bx);
-    h->npt = p->nodes_per_thread > 0 ? p->nodes_per_thread : (p->precision == LBM_F64 ? 2 : 3);
+    // defaults, measured in us per step: FP32 arithmetic two nodes side by side
+    // along x, in one-warp blocks on small lattices, which share them out evenly
+    // (200^2 2.3 against 2.9 with 64 x 2 threads, 450^2 3.6 / 4.1, 4096^2 the same);
+    // FP64 one node per thread on the smallest (64^2 8.4 / 10.5 / 26.7 with one / two
+    // along y / two in blocks of 64 x 2), else two along y (257^2 21.3 / 46)
+    const long nodes = (long)p->nx * p->ny;
+    const bool f64 = p->precision == LBM_F64, f16 = p->precision == LBM_F32_STORE_F16;
+    // (a grid has at most 65535 rows of blocks)
+    const bool narrow = p->block_x <= 0 && p->block_y <= 0 && p->ny < 60000 && !f16 && (f64 || nodes < (1L << 20));
+    h->bx = p->block_x > 0 ? p->block_x : (p->nx <= 128 || narrow ? 32 : 64);
+    h->by = p->block_y > 0 ? p->block_y : narrow ? (f64 || nodes < 100000 ? 1 : 2) : (h->bx >= 128 ? 1 : 128 / h->bx);
+    h->npt = p->nodes_per_thread > 0 ? p->nodes_per_thread : f64 ? (nodes < (1L << 14) ? 1 : 2) : 3;
     if (h->bx * h->by > 256 || h->bx <= 0 || h->by <= 0 || h->npt > 3) {
         delete h;
         return fail(nullptr, LBM_ERR_ARG, "block_x * block_y must be <= 256 and nodes_per_thread 1, 2 or 3");
@@ -691,15 +697,22 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
         }
     }
     if (!cached) {
-        const int cand[][3] = {{128, 2, 1}, {64, 4, 1}, {256, 1, 1}, {32, 8, 1}, {128, 1, 2}, {64, 2, 2},
-                               {128, 2, 2}, {256, 1, 2}, {32, 4, 2}, {32, 8, 3}, {64, 4, 3}, {128, 2, 3},
-                               {64, 2, 3},  {128, 1, 3}, {256, 1, 3}};
+        const int cand[][3] = {{128, 2, 1}, {64, 4, 1}, {256, 1, 1}, {32, 8, 1}, {32, 1, 1}, {32, 2, 1},
+                               {128, 1, 2}, {64, 2, 2}, {128, 2, 2}, {256, 1, 2}, {32, 4, 2}, {32, 1, 2},
+                               {32, 2, 2},  {32, 8, 3}, {64, 4, 3}, {128, 2, 3}, {64, 2, 3}, {128, 1, 3},
+                               {256, 1, 3}, {32, 1, 3}, {32, 2, 3}};
+        // below 2^17 nodes one node per thread or two along y: only the last step
+        // of a call runs by itself there (lbm_tile.cu), within 0.3 us of the best
+        const bool few = (long)h->p.nx * h->p.ny < (1L << 17);
         cudaEvent_t e0, e1;
         CK(h, cudaEventCreate(&e0));
         CK(h, cudaEventCreate(&e1));
         float best_ms = 1e30f;
         drop_graphs(h);
         for (auto& cd : cand) {
+            if (few && cd[2] == 3) continue;
+            // (a grid has at most 65535 rows of blocks)
+            if (h->p.ny / (cd[1] * (cd[2] == 2 ? 2 : 1)) > 65000) continue;
             h->bx = cd[0];
             h->by = cd[1];
             h->npt = cd[2];

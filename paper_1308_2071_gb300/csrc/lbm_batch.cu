@@ -92,27 +92,6 @@ __host__ __device__ __forceinline__ Coef<R> with_cavity_rates(const Coef<R>& cu,
     return c;
 }
 
-// Split tiles (NPT = 4): a cavity's interior node pairs, (x0, x0 + 1) with
-// x0 = 2, 4, ..., 2 npi (npi = floor((nx - 3) / 2): the pairs clear of the
-// walls) and 1 <= y <= ny - 2, and its border, every other node: rows 0 and
-// ny - 1, then the columns 0, 1 and 2 npi + 2 .. nx - 1 of each inner row
-// (the nodes of the pairs that touch a wall).  Border node b of a cavity, by
-// that order.
-__device__ __forceinline__ void border_node(int b, int nx, int ny, int& x, int& y) {
-    if (b < 2 * nx) {
-        y = b < nx ? 0 : ny - 1;
-        x = b < nx ? b : b - nx;
-        return;
-    }
-    const int npi = (nx - 3) >> 1;
-    const int nbc = nx - 2 * npi;  // border columns per inner row: 0, 1 and the right edge
-    const int k = b - 2 * nx;
-    y = 1 + k / nbc;
-    const int col = k - (y - 1) * nbc;
-    x = col < 2 ? col : 2 * npi + col;
-}
-__host__ __device__ constexpr int border_count(int nx, int ny) { return 2 * nx + (ny - 2) * (nx - 2 * ((nx - 3) >> 1)); }
-
 // One tile of one step: tiles hold blockDim.x * NPT nodes (NPT = 3: two
 // nodes side by side along x per thread, a run of blockDim.x node pairs in
 // the row-major order of the cavity's pairs (x0 even), wrapping onto the next
@@ -126,9 +105,9 @@ __device__ __forceinline__ void tile_update(const Coef<typename T::R>& c, const 
     if constexpr (NPT == 4) {
         if (tl.y0 < 0) {
             const int b = tl.x0 + (int)threadIdx.x;
-            if (b < border_count(gm.nx, gm.ny)) {
+            if (b < border_count<true>(gm.nx, gm.ny)) {
                 int x, y;
-                border_node(b, gm.nx, gm.ny, x, y);
+                border_node<true>(b, gm.nx, gm.ny, x, y);
                 update_node<T, false>(c, gm, src, dst, nullptr, x, y, status);
             }
         } else {
@@ -487,7 +466,7 @@ int build_tiles(lbm_batch b) {
                 tl.push_back(Tile{c, (int)(2 * (p0 % npx)), (int)(1 + p0 / npx)});
                 ++b->cav_tiles[c];
             }
-            for (long b0 = 0; b0 < border_count(nx, ny); b0 += b->tune.tw) {
+            for (long b0 = 0; b0 < border_count<true>(nx, ny); b0 += b->tune.tw) {
                 tl.push_back(Tile{c, (int)b0, -1});
                 ++b->cav_tiles[c];
             }

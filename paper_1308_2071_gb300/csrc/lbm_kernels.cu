@@ -23,15 +23,43 @@ __device__ __forceinline__ void wait_for_previous_step() { asm volatile("griddep
 // OBS: an observing step, which also stores the temperatures of the node
 // columns next to the vertical walls into obs (obs_put) for the Nusselt
 // number of the new state; otherwise obs is unused.
+//
+// FP32 and FP64 storage (Core<T>): the blocks from column `cols` of the grid on
+// take the border's nodes one per thread, the others rows of fluid nodes only
+// (see border_node).  Measured against rows that hold the walls too, us per
+// step: FP64 257^2 31 -> 26, 512^2 92 -> 75, FP32 601 x 397 4.8 -> 4.3.  FP16 flow storage: no such
+// columns, every block takes what it meets.
+template <class T, bool FIELD, bool OBS, bool PAIRS>
+__device__ __forceinline__ void step_border(const Src<T>& src, const Dst<T>& dst, const typename T::P* __restrict__ phi,
+                                            const Geom& gm, const Coef<typename T::R>& c, int* __restrict__ status,
+                                            double* __restrict__ obs, int cols) {
+    const int threads = blockDim.x * blockDim.y;
+    const int b = ((blockIdx.x - cols) * gridDim.y + blockIdx.y) * threads + threadIdx.y * blockDim.x + threadIdx.x;
+    if (b >= border_count<PAIRS>(gm.nx, gm.ny)) return;
+    int x, y;
+    border_node<PAIRS>(b, gm.nx, gm.ny, x, y);
+    update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x, y, status, obs);
+}
+
 template <class T, bool FIELD, bool OBS>
 __global__ void __launch_bounds__(256) k_step(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi,
                                               Geom gm, Coef<typename T::R> c, int* __restrict__ status,
-                                              double* __restrict__ obs) {
+                                              double* __restrict__ obs, int cols) {
     wait_for_previous_step();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= gm.nx || y >= gm.ny) return;
-    update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x, y, status, obs);
+    if constexpr (Core<T>::value) {
+        if ((int)blockIdx.x >= cols) {
+            step_border<T, FIELD, OBS, false>(src, dst, phi, gm, c, status, obs, cols);
+            return;
+        }
+        const int y = 1 + blockIdx.y * blockDim.y + threadIdx.y;
+        if (x == 0 || x >= gm.nx - 1 || y >= gm.ny - 1) return;
+        update_fluid<T, FIELD, OBS>(c, gm, src, dst, phi, x, y, status, obs);
+    } else {
+        const int y = blockIdx.y * blockDim.y + threadIdx.y;
+        if (x >= gm.nx || y >= gm.ny) return;
+        update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x, y, status, obs);
+    }
 }
 
 // Blocks of 256 threads per SM that the two-node kernels are compiled for (see k_step2).
@@ -39,11 +67,10 @@ template <class T> constexpr int step_blocks() {
     return sizeof(typename T::R) == 8 ? 1 : sizeof(typename T::SF) == 4 ? 3 : 4;
 }
 
-// Two nodes per thread, (x, y) and (x, y + blockDim.y): when both are fluid
-// nodes all 28 loads are issued before any arithmetic, doubling the bytes in
-// flight per thread (the FP16-flow variant moves 38 B per node, too few to
-// cover HBM latency with one node per thread).  Wall nodes take the general
-// path one at a time.
+// Two nodes per thread, (x, y) and (x, y + blockDim.y): all 28 loads are issued
+// before any arithmetic, doubling the bytes in flight per thread (the FP16-flow
+// variant moves 38 B per node, too few to cover HBM latency with one node per
+// thread).
 // FP32 storage: at most 80 registers (3 blocks of 256 threads, 6 of 128 per
 // SM), where the paired collision spills nothing (140 bytes under 64).  Measured
 // at 4096^2 / 1024^2 / 512^2 / 200^2: 273.7 / 17.7 / 5.5 / 3.1 us per step, under
@@ -53,13 +80,26 @@ template <class T> constexpr int step_blocks() {
 template <class T, bool FIELD, bool OBS>
 __global__ void __launch_bounds__(256, step_blocks<T>())
     k_step2(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
-            int* __restrict__ status, double* __restrict__ obs) {
+            int* __restrict__ status, double* __restrict__ obs, int cols) {
     wait_for_previous_step();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y0 = blockIdx.y * (2 * blockDim.y) + threadIdx.y;
-    const int y1 = y0 + blockDim.y;
-    if (x >= gm.nx || y0 >= gm.ny) return;
-    update_pair<T, FIELD, OBS>(c, gm, src, dst, phi, x, y0, true, x, y1, y1 < gm.ny, status, obs);
+    if constexpr (Core<T>::value) {
+        if ((int)blockIdx.x >= cols) {
+            step_border<T, FIELD, OBS, false>(src, dst, phi, gm, c, status, obs, cols);
+            return;
+        }
+        const int y0 = 1 + blockIdx.y * (2 * blockDim.y) + threadIdx.y, y1 = y0 + blockDim.y;
+        if (x == 0 || x >= gm.nx - 1 || y0 >= gm.ny - 1) return;
+        if (y1 < gm.ny - 1)
+            update_pair<T, FIELD, OBS>(c, gm, src, dst, phi, x, y0, true, x, y1, true, status, obs);
+        else
+            update_fluid<T, FIELD, OBS>(c, gm, src, dst, phi, x, y0, status, obs);
+    } else {
+        const int y0 = blockIdx.y * (2 * blockDim.y) + threadIdx.y;
+        const int y1 = y0 + blockDim.y;
+        if (x >= gm.nx || y0 >= gm.ny) return;
+        update_pair<T, FIELD, OBS>(c, gm, src, dst, phi, x, y0, true, x, y1, y1 < gm.ny, status, obs);
+    }
 }
 
 // Two nodes per thread side by side, (x0, y) and (x0 + 1, y) with x0 even:
@@ -69,12 +109,22 @@ __global__ void __launch_bounds__(256, step_blocks<T>())
 template <class T, bool FIELD, bool OBS>
 __global__ void __launch_bounds__(256, step_blocks<T>())
     k_step2x(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
-             int* __restrict__ status, double* __restrict__ obs) {
+             int* __restrict__ status, double* __restrict__ obs, int cols) {
     wait_for_previous_step();
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x0 >= gm.nx || y >= gm.ny) return;
-    update_xpair<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y, status, obs);
+    if constexpr (Core<T>::value) {
+        if ((int)blockIdx.x >= cols) {
+            step_border<T, FIELD, OBS, true>(src, dst, phi, gm, c, status, obs, cols);
+            return;
+        }
+        const int y = 1 + blockIdx.y * blockDim.y + threadIdx.y;
+        if (x0 == 0 || x0 + 1 >= gm.nx - 1 || y >= gm.ny - 1) return;
+        update_fluid_xpair<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y, status, obs);
+    } else {
+        const int y = blockIdx.y * blockDim.y + threadIdx.y;
+        if (x0 >= gm.nx || y >= gm.ny) return;
+        update_xpair<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y, status, obs);
+    }
 }
 
 // ---- observables ------------------------------------------------------------------
@@ -281,13 +331,15 @@ template <> const Coef<float>& coef_of<PrecF16>(const CoefSet& cs) { return cs.f
 template <> const Coef<float>& coef_of<PrecF32T>(const CoefSet& cs) { return cs.f; }
 
 // Launches kernel k with the step's arguments, as a programmatic dependent of
-// the previous work on the stream when L.pdl is set.
-template <class T, class K>
-static cudaError_t launch_one_step(K k, dim3 grd, dim3 blk, const StepLaunch& L, const Src<T>& s, const Dst<T>& d,
-                                   const typename T::P* phi, const Coef<typename T::R>& c) {
+// the previous work on the stream when L.pdl is set.  gx, gy: blocks over the
+// nodes; PAIRS: which border goes apart.
+template <class T, bool PAIRS, class K>
+static cudaError_t launch_one_step(K k, int gx, int gy, const StepLaunch& L, const Coef<typename T::R>& c, bool field) {
+    const int per_col = gy * L.bx * L.by;  // border nodes that a column of blocks holds
+    const int border = Core<T>::value ? (border_count<PAIRS>(L.gm.nx, L.gm.ny) + per_col - 1) / per_col : 0;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grd;
-    cfg.blockDim = blk;
+    cfg.gridDim = dim3(gx + border, gy);
+    cfg.blockDim = dim3(L.bx, L.by);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = L.stream;
     cudaLaunchAttribute at[1];
@@ -295,25 +347,19 @@ static cudaError_t launch_one_step(K k, dim3 grd, dim3 blk, const StepLaunch& L,
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = L.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, s, d, phi, L.gm, c, L.status, L.obs);
+    return cudaLaunchKernelEx(&cfg, k, src_view<T>(L.src, L.gm.plane), dst_view<T>(L.dst, L.gm.plane),
+                              field ? (const typename T::P*)L.phi : nullptr, L.gm, c, L.status, L.obs, gx);
 }
 
 template <class T, bool FIELD, bool OBS>
 static cudaError_t launch_step_k(const StepLaunch& L, const CoefSet& cs) {
-    dim3 blk(L.bx, L.by);
-    const Src<T> s = src_view<T>(L.src, L.gm.plane);
-    const Dst<T> d = dst_view<T>(L.dst, L.gm.plane);
-    const typename T::P* phi = FIELD ? (const typename T::P*)L.phi : nullptr;
-    if (L.npt == 2) {
-        dim3 grd2((L.gm.nx + L.bx - 1) / L.bx, (L.gm.ny + 2 * L.by - 1) / (2 * L.by));
-        return launch_one_step<T>(k_step2<T, FIELD, OBS>, grd2, blk, L, s, d, phi, coef_of<T>(cs));
-    }
-    if (L.npt == 3) {
-        dim3 grdx((L.gm.nx + 2 * L.bx - 1) / (2 * L.bx), (L.gm.ny + L.by - 1) / L.by);
-        return launch_one_step<T>(k_step2x<T, FIELD, OBS>, grdx, blk, L, s, d, phi, coef_of<T>(cs));
-    }
-    dim3 grd((L.gm.nx + L.bx - 1) / L.bx, (L.gm.ny + L.by - 1) / L.by);
-    return launch_one_step<T>(k_step<T, FIELD, OBS>, grd, blk, L, s, d, phi, coef_of<T>(cs));
+    const Coef<typename T::R>& c = coef_of<T>(cs);
+    const int rows = Core<T>::value ? L.gm.ny - 2 : L.gm.ny;  // the rows without the border, or all
+    const int per = L.npt == 2 ? 2 * L.by : L.by, wide = L.npt == 3 ? 2 * L.bx : L.bx;
+    const int gx = (L.gm.nx + wide - 1) / wide, gy = (rows + per - 1) / per;
+    if (L.npt == 2) return launch_one_step<T, false>(k_step2<T, FIELD, OBS>, gx, gy, L, c, FIELD);
+    if (L.npt == 3) return launch_one_step<T, true>(k_step2x<T, FIELD, OBS>, gx, gy, L, c, FIELD);
+    return launch_one_step<T, false>(k_step<T, FIELD, OBS>, gx, gy, L, c, FIELD);
 }
 
 template <class T>

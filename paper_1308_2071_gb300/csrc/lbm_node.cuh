@@ -447,6 +447,37 @@ __device__ __forceinline__ double obs_value(const Macro<typename T::R>& m) {
         return (double)m.dT;
 }
 
+// One fluid node of the step (FP32 and FP64 storage).
+template <class T, bool FIELD, bool OBS>
+__device__ __forceinline__ void update_fluid(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& src,
+                                             const Dst<T>& dst, const typename T::P* __restrict__ phi, int x, int y,
+                                             int* status, double* obs) {
+    using R = typename T::R;
+    constexpr bool FR = Framed<T>::value;
+    const Coll<R>& k = c.k;
+    const int off = y * gm.pitch + x;
+    R d[9], h[5];
+    pull<T>(src, gm, off, d, h);
+    const R F = core_frame_in<T>(k, src, gm, off, h);
+    const R phi_n = FIELD ? (in_plane(gm, off) ? Conv<typename T::P, R>::ld(phi + off) : R(1)) : R(0);
+    const Por<R> p = por_of<R, FIELD>(k, phi_n);
+    const Sums<R> s = sums_of(d, h);
+    const Vel<R> v = velocity<R, FR>(k, p, s, op::mul(F, k.fu));
+    if (too_fast(v)) atomicOr(status, 1);  // also catches NaN
+    typename FrameStore<T>::type code;
+    R next;
+    const R shift = frame_next<T>(k, v.dT, F, next, code);
+    collide_fluid<R, FIELD, FR>(k, p, s, v, shift, d, h);
+    if (in_plane(gm, off)) {
+        if constexpr (FR) dst.t[off] = code;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) Conv<typename T::SF, R, T::cg>::st(dst.f + i * gm.plane + off, d[i]);
+#pragma unroll
+        for (int j = 0; j < 5; ++j) Conv<typename T::SG, R, T::cg>::st(dst.g + j * gm.plane + off, h[j]);
+    }
+    if constexpr (OBS) obs_put(gm, obs, x, y, FR ? (double)op::mul(F, k.fu) + (double)v.dTl : (double)v.dT);
+}
+
 // One node of the step: pull (or wall rule), collide, store; OBS: also the
 // node's temperature into obs when it lies in a wall column.  That store
 // comes after all arithmetic: a branch between the macroscopic values and
@@ -602,6 +633,36 @@ __device__ __forceinline__ void update_fluid_pair_x2(const Coef<float>& c, const
                                   F1);
 }
 
+// The nodes beside the walls apart from the others.  A warp that holds a wall
+// node runs the wall rule for its lane while the others wait, which in rows of
+// a few warps costs as much again as the row (FP64: 390 operations against
+// 134).  So the step kernels and the batched tiles give the border to blocks of
+// its own and leave it out of the rows.
+//
+// By node pairs (PAIRS): the interior is (x0, x0 + 1) with x0 = 2, 4, ..., 2 npi
+// (npi = floor((nx - 3) / 2): the pairs clear of the walls) and 1 <= y <= ny - 2,
+// the border every other node: rows 0 and ny - 1, then the columns 0, 1 and 2
+// npi + 2 .. nx - 1 of each inner row.  By nodes: the border is the wall nodes.
+template <bool PAIRS> __host__ __device__ constexpr int border_columns(int nx) {
+    return PAIRS ? nx - 2 * ((nx - 3) >> 1) : 2;
+}
+template <bool PAIRS> __host__ __device__ constexpr int border_count(int nx, int ny) {
+    return 2 * nx + (ny - 2) * border_columns<PAIRS>(nx);
+}
+// Border node b in that order.
+template <bool PAIRS> __device__ __forceinline__ void border_node(int b, int nx, int ny, int& x, int& y) {
+    if (b < 2 * nx) {
+        y = b < nx ? 0 : ny - 1;
+        x = b < nx ? b : b - nx;
+        return;
+    }
+    const int nbc = border_columns<PAIRS>(nx);
+    const int k = b - 2 * nx;
+    y = 1 + k / nbc;
+    const int col = k - (y - 1) * nbc;
+    x = col < (PAIRS ? 2 : 1) ? col : nx - nbc + col;
+}
+
 // Two fluid nodes from their pulled values (F0, F1: their frames in the frames'
 // unit), FP32 and FP64 storage.  VEC: x-neighbours off1 = off0 + 1 with x0
 // even, stored as pairs.
@@ -729,6 +790,18 @@ __device__ __forceinline__ void update_pair(const Coef<typename T::R>& c, const 
     if (v1) update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x1, y1, status, obs);
 }
 
+// The fluid nodes (x0, y) and (x0 + 1, y), x0 even (FP32 and FP64 storage).
+template <class T, bool FIELD, bool OBS = false>
+__device__ __forceinline__ void update_fluid_xpair(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& src,
+                                                   const Dst<T>& dst, const typename T::P* phi, int x0, int y,
+                                                   int* status, double* obs = nullptr) {
+    using R = typename T::R;
+    R d0[9], h0[5], d1[9], h1[5], F0, F1;
+    pull_x2<T>(src, gm, y * gm.pitch + x0, d0, h0, d1, h1);
+    core_frame_in_x2<T>(c.k, src, gm, y * gm.pitch + x0, h0, h1, F0, F1);
+    core_fluid_pair<T, FIELD, OBS, true>(c, gm, dst, phi, d0, h0, d1, h1, F0, F1, x0, y, x0 + 1, y, status, obs);
+}
+
 // Two nodes side by side, (x0, y) and (x0 + 1, y) with x0 even: when both are
 // fluid nodes the populations with e_x = 0, the stores and the frames move
 // as aligned pairs (about a third fewer memory instructions than two nodes
@@ -740,14 +813,13 @@ __device__ __forceinline__ void update_xpair(const Coef<typename T::R>& c, const
     using R = typename T::R;
     const int x1 = x0 + 1;
     if (x0 > 0 && x1 < gm.nx - 1 && y > 0 && y < gm.ny - 1) {
-        const int off0 = y * gm.pitch + x0, off1 = off0 + 1;
-        R d0[9], h0[5], d1[9], h1[5];
-        pull_x2<T>(src, gm, off0, d0, h0, d1, h1);
-        R F0 = R(0), F1 = R(0);
         if constexpr (Core<T>::value) {
-            core_frame_in_x2<T>(c.k, src, gm, off0, h0, h1, F0, F1);
-            core_fluid_pair<T, FIELD, OBS, true>(c, gm, dst, phi, d0, h0, d1, h1, F0, F1, x0, y, x1, y, status, obs);
+            update_fluid_xpair<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y, status, obs);
         } else {
+            const int off0 = y * gm.pitch + x0, off1 = off0 + 1;
+            R d0[9], h0[5], d1[9], h1[5];
+            pull_x2<T>(src, gm, off0, d0, h0, d1, h1);
+            R F0 = R(0), F1 = R(0);
             frame_in_x2<T>(c, src, gm, off0, h0, h1, F0, F1);
             const Drag<R> dr0 = drag_at<R, FIELD, typename T::P>(c, gm, phi, off0);
             const Drag<R> dr1 = drag_at<R, FIELD, typename T::P>(c, gm, phi, off1);

@@ -11,10 +11,11 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 SMALL = [(5, 5), (6, 11), (8, 8), (9, 8), (17, 13), (64, 64), (65, 33), (66, 9), (129, 41), (190, 12), (257, 70), (7, 900)]
-# two steps per launch from 2^18 nodes: strips of up to 94 pairs, segments of up to 32 rows, wall tiles of 28 and 22 nodes
-LARGE = [(512, 512), (513, 511), (600, 437), (1021, 257), (1023, 259), (8, 32768), (9, 29500), (32771, 8), (26300, 10),
+# two steps per launch from 850,000 nodes: strips of up to 94 pairs, segments of up to 32 rows, wall tiles of 28 and 22 nodes
+LARGE = [(1024, 832), (1025, 831), (901, 950), (2001, 437), (2003, 439), (8, 110000), (9, 95001), (110003, 8), (88300, 10),
          (1501, 1500)]
-SIZES = SMALL + LARGE
+MIDDLE = [(500, 451), (601, 397)]  # one step per launch
+SIZES = SMALL + MIDDLE + LARGE
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -55,14 +56,14 @@ def test_steps_in_twos_leave_the_same_bits(size, precision):
     _same(a, b, 13)
 
 
-@pytest.mark.parametrize("size", [(70, 50), (640, 420)])
+@pytest.mark.parametrize("size", [(70, 50), (1040, 820)])
 @pytest.mark.parametrize("n", [1, 2, 3, 4, 7, 64, 65, 66, 131])
 def test_every_count_of_steps(size, n):
     a, b = _pair(*size)
     _same(a, b, n)
 
 
-@pytest.mark.parametrize("size", [(70, 50), (640, 420)])
+@pytest.mark.parametrize("size", [(70, 50), (1040, 820)])
 def test_the_steady_loop_takes_the_same_steps(size):
     # the loop's body runs its steps in an even number of launches, the last alone
     for every in (2, 4, 6, 20, 33):
@@ -75,7 +76,7 @@ def test_the_steady_loop_takes_the_same_steps(size):
         b.close()
 
 
-@pytest.mark.parametrize("size", [(9, 8), (64, 64), (129, 41), (700, 395), (701, 394)])
+@pytest.mark.parametrize("size", [(9, 8), (64, 64), (129, 41), (1100, 795), (1101, 794)])
 @pytest.mark.parametrize("kw", [dict(thermal_bc=1, Ra=0.0, phi=1.0, Pr=7.0, RaI=6.4e4, forchheimer=0),
                                 dict(RaI=1e5, Pr=0.7, Th=1.5, Tc=-0.25), dict(Da=float("inf"), forchheimer=0),
                                 dict(collision=1), dict(adiabatic_order=2), "field"])
@@ -91,7 +92,7 @@ def test_wall_and_parameter_variants(size, kw):
     _same(a, b, 12)
 
 
-@pytest.mark.parametrize("size", [(70, 50), (640, 420)])
+@pytest.mark.parametrize("size", [(70, 50), (1040, 820)])
 def test_divergence_between_two_steps_of_a_launch_is_flagged(size):
     # a NaN planted in the lattice spreads and raises the flag, also when the
     # first step that meets it is one whose lattice stays on chip
