@@ -1,6 +1,7 @@
-// Batched sweep: many cavities of different size and parameters advanced by
-// one persistent kernel launch that runs every requested step, captured once
-// into a CUDA graph and replayed.  Each block walks a flat list of tiles
+// Batched sweep: many cavities of different size and parameters advanced
+// together, either by one persistent kernel launch that runs every requested
+// step, captured once into a CUDA graph and replayed, or, where the autotuner
+// finds that faster, two steps per launch (k_batch_duo) before the last ones.  Each block walks a flat list of tiles
 // covering every cavity; a grid-wide barrier separates the steps (each step
 // reads the whole previous lattice of its cavity).  The per-node work is the
 // same device code as the single-cavity step kernel, so a cavity advanced
@@ -15,6 +16,7 @@
 #include <string>
 #include <vector>
 
+#include "lbm_duo.cuh"
 #include "lbm_internal.h"
 #include "lbm_sync.cuh"
 
@@ -22,10 +24,13 @@ using namespace lbm;
 
 namespace lbm {
 
+constexpr int kDuoThreads = 128;  // of a block that takes two steps of a cavity at once
+
 template <class R> struct CavDesc {
     Geom gm;
     void* buf[2];  // B_n / B_{n+1} ping-pong of this cavity
     int ntiles;    // tiles covering this cavity
+    int strips, width, rows;  // two steps per launch: strips of node pairs, rows per segment
     Coef<R> c;
 };
 
@@ -305,6 +310,35 @@ __global__ void __launch_bounds__(256, sizeof(typename T::R) == 4 ? 3 : 2)
     }
 }
 
+// Two steps of every cavity (lbm_duo.cuh): block i does work[i] = (cavity, march
+// of it, or -1 - wall tile).  Nothing waits inside: the steps of a pair meet in
+// shared memory, pairs of steps are launches.  FP32 storage with batch-wide
+// coefficients in cu (SPLIT, see k_batch).  Measured on the 256-cavity sweep, us
+// per step: persistent kernel 490, this 327, of which the wall tiles 45 (they read
+// and write narrow columns; as a launch of their own in 64 registers 75, mixed
+// with the marches 50).  Blocks of 64 / 96 / 128 threads: 339 / 353 / 327.
+template <class T>
+__global__ void __launch_bounds__(kDuoThreads, 512 / kDuoThreads)
+    k_batch_duo(const CavDesc<float>* __restrict__ cavs, const int2* __restrict__ work, int par,
+                int* __restrict__ status, const __grid_constant__ Coef<float> cu) {
+    __shared__ float2 sh[kDuoRows * (kDuoThreads + 2)];
+    __shared__ CavDesc<float> cd;
+    const int2 w = work[blockIdx.x];
+    for (int k = threadIdx.x; k < (int)(sizeof(CavDesc<float>) / sizeof(int)); k += kDuoThreads)
+        ((int*)&cd)[k] = ((const int*)&cavs[w.x])[k];
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the previous launch is complete
+    __syncthreads();
+    const Geom gm = cd.gm;
+    const Coef<float> c = with_cavity_rates(cu, cd.c);
+    const Src<T> src = src_view<T>(cd.buf[par], gm.plane);
+    const Dst<T> dst = dst_view<T>(cd.buf[par ^ 1], gm.plane);
+    if (w.y >= 0)
+        duo_march_block<T, false, kDuoThreads>(w.y, src, dst, nullptr, gm, c.k, &status[w.x], cd.strips, cd.width,
+                                               cd.rows, sh);
+    else
+        duo_wall_block<T, false, kDuoThreads>(-1 - w.y, src, dst, nullptr, gm, c, &status[w.x], (float*)sh);
+}
+
 // Mean Nusselt numbers (Eq. 38) of every cavity, one block per cavity, FP64.
 template <class T>
 __global__ void __launch_bounds__(256) k_batch_nusselt(const CavDesc<typename T::R>* __restrict__ cavs,
@@ -361,8 +395,13 @@ namespace {
 constexpr long long kDefaultWaitPolls = 20000000;  // ~2-20 s of 100 ns polls
 
 // th = 0: linear tiles, runs of tw consecutive nodes in row-major order
+// dyn: the schedule of the persistent kernel (0 to 2), plus kInTwos when the
+// steps run two per launch and the persistent kernel takes the last ones.
+constexpr int kInTwos = 3;
 struct TuneChoice {
     int tw = 128, th = 2, blocks_per_sm = 0, dyn = 0;
+    int schedule() const { return dyn % kInTwos; }
+    bool in_twos() const { return dyn >= kInTwos; }
 };
 
 // th = -1: runs of tw node pairs (two nodes side by side along x per thread);
@@ -389,6 +428,8 @@ struct lbm_batch_s {
     void* descs = nullptr;  // CavDesc<R>[ncav]
     Tile* tiles = nullptr;
     int ntiles = 0;
+    int2* work = nullptr;  // two steps per launch: (cavity, block) of every block; nullptr where it does not run
+    int nwork = 0;
     double* Ls = nullptr;   // (L, dT) per cavity
     double* nu_dev = nullptr;
     int* status = nullptr;  // per cavity
@@ -520,7 +561,7 @@ int launch(lbm_batch b, long nsteps, int par, cudaStream_t s) {
     int lg = b->tune.th <= 0 ? -1 : log2i(b->tune.tw), nt = b->ntiles;
     const void* descs = b->descs;
     const Tile* tiles = b->tiles;
-    int dyn = b->tune.dyn;
+    int dyn = b->tune.schedule();
     args[0] = &descs;
     args[1] = &tiles;
     args[2] = &nt;
@@ -538,13 +579,71 @@ int launch(lbm_batch b, long nsteps, int par, cudaStream_t s) {
     Coef<double> cud = b->coef[0].d;
     args[13] = b->precision == LBM_F64 ? (void*)&cud : (void*)&cuf;
     cudaError_t ez = cudaMemsetAsync(b->tile_ctr, 0, 2 * sizeof(int), s);
-    if (ez == cudaSuccess && b->tune.dyn == 2)  // finished-tile counters of the dataflow mode
+    if (ez == cudaSuccess && dyn == 2)  // finished-tile counters of the dataflow mode
         ez = cudaMemsetAsync(b->bar + 2, 0, sizeof(unsigned) * (size_t)b->ncav, s);
     if (ez != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("counter reset: ") + cudaGetErrorString(ez));
     const int npt = npt_of(b->tune);
     const void* k = batch_kernel(b->precision, npt, b->split);
     cudaError_t e = cudaLaunchCooperativeKernel(k, dim3(b->nblocks), dim3(block_of(b->tune)), args, 0, s);
     if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("cooperative launch: ") + cudaGetErrorString(e));
+    return LBM_OK;
+}
+
+// The march of one cavity: strips as wide as fill the block's warps best, and
+// segments of at most 48 rows (32: 331 us per step of the sweep, 48: 327).
+bool duo_layout(const Geom& gm, int* strips, int* width, int* rows) {
+    *strips = *width = *rows = 0;
+    if (gm.nx < 8 || gm.ny < 8 || gm.adi_order != 1) return false;
+    const int pairs = duo_last_pair(gm.nx) - duo_first_pair() + 1, inner = gm.ny - 4;
+    long best = 1L << 60;
+    const int least = (pairs + kDuoThreads - 3) / (kDuoThreads - 2);
+    for (int n = least; n <= least + 2 && n <= pairs; ++n) {
+        const int w = (pairs + n - 1) / n, used = (pairs + w - 1) / w;
+        const long warps = (long)used * ((w + 2 + 31) / 32);
+        if (warps < best) {
+            best = warps;
+            *strips = used;
+            *width = w;
+        }
+    }
+    const int segs = (inner + 47) / 48;
+    *rows = (inner + segs - 1) / segs;
+    return true;
+}
+
+// The blocks of the two-step launch: the marches, then the (shorter) wall
+// tiles.  None where a cavity does not qualify or the coefficients are
+// not batch-wide.
+int build_work(lbm_batch b) {
+    if (b->precision == LBM_F64 || !b->split) return LBM_OK;
+    std::vector<int2> march, walls;
+    for (int c = 0; c < b->ncav; ++c) {
+        int strips, width, rows;
+        if (!duo_layout(b->gm[c], &strips, &width, &rows)) return LBM_OK;
+        const int nt = duo_tiles(b->gm[c].nx, b->gm[c].ny, kDuoThreads), segs = (b->gm[c].ny - 4 + rows - 1) / rows;
+        for (int i = 0; i < nt; ++i) walls.push_back(make_int2(c, -1 - i));
+        for (int i = 0; i < strips * segs; ++i) march.push_back(make_int2(c, i));
+    }
+    march.insert(march.end(), walls.begin(), walls.end());
+    BCK(b, cudaMalloc(&b->work, sizeof(int2) * march.size()));
+    BCK(b, cudaMemcpy(b->work, march.data(), sizeof(int2) * march.size(), cudaMemcpyHostToDevice));
+    b->nwork = (int)march.size();
+    return LBM_OK;
+}
+
+int launch_twos(lbm_batch b, int par, bool pdl, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kDuoThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    const CavDesc<float>* descs = (const CavDesc<float>*)b->descs;
+    cfg.gridDim = dim3(b->nwork);
+    cfg.numAttrs = pdl ? 1 : 0;
+    BCK(b, cudaLaunchKernelEx(&cfg, b->precision == LBM_F32_FRAMED ? k_batch_duo<PrecF32T> : k_batch_duo<PrecF32Q>,
+                              descs, (const int2*)b->work, par, b->status, b->coef[0].f));
     return LBM_OK;
 }
 
@@ -555,6 +654,7 @@ template <class R> int upload_descs(lbm_batch b) {
         h[c].buf[0] = (char*)b->pool + b->off[0][c];
         h[c].buf[1] = (char*)b->pool + b->off[1][c];
         h[c].ntiles = c < (int)b->cav_tiles.size() ? b->cav_tiles[c] : 0;
+        duo_layout(b->gm[c], &h[c].strips, &h[c].width, &h[c].rows);
         if constexpr (sizeof(R) == 8) h[c].c = b->coef[c].d;
         else h[c].c = b->coef[c].f;
     }
@@ -593,6 +693,12 @@ void drop_graph(lbm_batch b) {
 
 int run_steps(lbm_batch b, long nsteps, cudaStream_t s) {
     if (nsteps <= 0) return LBM_OK;
+    // two per launch, but for the last one or two steps, which leave B_{n-1}
+    for (bool first = true; b->tune.in_twos() && nsteps >= 3; nsteps -= 2, first = false) {
+        int rc = launch_twos(b, b->par, !first, s);
+        if (rc != LBM_OK) return rc;
+        b->par ^= 1;
+    }
     const int par = b->par;
     if (!(b->gexec && b->gexec_steps == nsteps && b->gexec_par == par && b->gexec_limit == b->wait_limit)) {
         drop_graph(b);
@@ -724,6 +830,7 @@ int lbm_batch_init(const lbm_params* p, int ncav, void* stream, lbm_batch* out) 
     if (cudaMemcpy(b->Ls, Ls.data(), sizeof(double) * 2 * ncav, cudaMemcpyHostToDevice) != cudaSuccess)
         rc = bfail(b, LBM_ERR_CUDA, "parameter upload");
     if (rc == LBM_OK) rc = prec == LBM_F64 ? upload_descs<double>(b) : upload_descs<float>(b);
+    if (rc == LBM_OK) rc = build_work(b);
     if (rc == LBM_OK) rc = build_tiles(b);
     if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
     if (rc == LBM_OK) rc = reset(b);
@@ -834,34 +941,47 @@ int lbm_batch_tune(lbm_batch b, const char* cache_path, int* tile_w, int* tile_h
         BCK(b, cudaEventCreate(&e0));
         BCK(b, cudaEventCreate(&e1));
         const long nsteps = 20;
+        // times b->tune and keeps it if it is the best so far
+        auto trial = [&]() -> int {
+            int rc = build_tiles(b);
+            if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
+            drop_graph(b);
+            if (rc == LBM_OK) rc = run_steps(b, 2, b->stream);  // warm
+            if (rc != LBM_OK) return rc;
+            BCK(b, cudaEventRecord(e0, b->stream));
+            rc = run_steps(b, nsteps, b->stream);
+            if (rc != LBM_OK) return rc;
+            BCK(b, cudaEventRecord(e1, b->stream));
+            BCK(b, cudaEventSynchronize(e1));
+            float ms = 0.f;
+            BCK(b, cudaEventElapsedTime(&ms, e0, e1));
+            if (ms < best_ms) {
+                best_ms = ms;
+                best = b->tune;
+            }
+            return LBM_OK;
+        };
         for (auto& sh : shapes)
             for (int o : occ)
-            for (int dyn = 0; dyn < 3; ++dyn) {
-                b->tune.tw = sh[0];
-                b->tune.th = sh[1];
-                b->tune.blocks_per_sm = o;
-                b->tune.dyn = dyn;
-                int rc = build_tiles(b);
-                if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
-                drop_graph(b);
-                if (rc == LBM_OK) rc = run_steps(b, 2, b->stream);  // warm
-                if (rc != LBM_OK) return rc;
-                BCK(b, cudaEventRecord(e0, b->stream));
-                rc = run_steps(b, nsteps, b->stream);
-                if (rc != LBM_OK) return rc;
-                BCK(b, cudaEventRecord(e1, b->stream));
-                BCK(b, cudaEventSynchronize(e1));
-                float ms = 0.f;
-                BCK(b, cudaEventElapsedTime(&ms, e0, e1));
-                if (ms < best_ms) {
-                    best_ms = ms;
-                    best = b->tune;
+                for (int dyn = 0; dyn < kInTwos; ++dyn) {
+                    b->tune.tw = sh[0];
+                    b->tune.th = sh[1];
+                    b->tune.blocks_per_sm = o;
+                    b->tune.dyn = dyn;
+                    int rc = trial();
+                    if (rc != LBM_OK) return rc;
                 }
-            }
+        if (b->work) {  // two steps per launch before that
+            b->tune = best;
+            b->tune.dyn += kInTwos;
+            int rc = trial();
+            if (rc != LBM_OK) return rc;
+        }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         if (cache_path) cache_store(cache_path, b->signature, best);
     }
+    if (best.dyn < 0 || (best.in_twos() && !b->work)) best.dyn = best.dyn < 0 ? 0 : best.schedule();
     b->tune = best;
     int rc = build_tiles(b);
     if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
@@ -911,6 +1031,7 @@ int lbm_batch_destroy(lbm_batch b) {
     if (b->pool) cudaFree(b->pool);
     if (b->descs) cudaFree(b->descs);
     if (b->tiles) cudaFree(b->tiles);
+    if (b->work) cudaFree(b->work);
     if (b->Ls) cudaFree(b->Ls);
     if (b->nu_dev) cudaFree(b->nu_dev);
     if (b->status) cudaFree(b->status);
