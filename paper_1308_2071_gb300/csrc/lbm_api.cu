@@ -809,6 +809,7 @@ int lbm_observables(lbm_handle h, lbm_obs* out, void* ux_dev, void* uy_dev, void
     L.dT = h->dv.dT;
     L.status = h->status_dev;
     L.out = h->obs_dev;
+    L.counter = h->nu_counter;
     L.stream = h->stream;
     CK(h, launch_observe(L, h->coef));
     CK(h, cudaMemcpyAsync(h->obs_host, h->obs_dev, sizeof(double) * 7, cudaMemcpyDeviceToHost, h->stream));

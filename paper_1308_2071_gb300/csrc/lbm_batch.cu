@@ -1,11 +1,12 @@
 // Batched sweep: many cavities of different size and parameters advanced
 // together, either by one persistent kernel launch that runs every requested
 // step, captured once into a CUDA graph and replayed, or, where the autotuner
-// finds that faster, two steps per launch (k_batch_duo) before the last ones.  Each block walks a flat list of tiles
-// covering every cavity; a grid-wide barrier separates the steps (each step
-// reads the whole previous lattice of its cavity).  The per-node work is the
-// same device code as the single-cavity step kernel, so a cavity advanced
-// here matches the same cavity advanced alone bit for bit.
+// finds that faster, two steps per launch (k_batch_duo) before the last ones.
+// In the persistent kernel each block walks a flat list of tiles covering every
+// cavity; a grid-wide barrier separates the steps (each step reads the whole
+// previous lattice of its cavity).  The per-node work is the same device code as
+// the single-cavity step kernel, so a cavity advanced here matches the same
+// cavity advanced alone bit for bit.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>

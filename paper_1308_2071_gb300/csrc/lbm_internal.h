@@ -93,7 +93,7 @@ struct ObserveLaunch {
     double L, dT;
     const int* status;
     double* out;            // 7 doubles
-    unsigned* counter = nullptr;  // launch_nusselt: zero-initialised block counter
+    unsigned* counter = nullptr;  // zero-initialised block counter (left at zero)
     const double* obs = nullptr;  // launch_nusselt: read the wall columns an observing step stored
     cudaStream_t stream;
 };

@@ -1,6 +1,8 @@
 // Kernels of the single-cavity path: the fused collide-and-stream step, the
-// observables pass, the final FP64 reductions with the Nusselt number, the
-// state export, and the porosity conversion.
+// observables pass with its FP64 reductions and the Nusselt number, the state
+// export, and the porosity conversion.
+#include <algorithm>
+
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -129,84 +131,123 @@ __global__ void __launch_bounds__(256, step_blocks<T>())
 
 // ---- observables ------------------------------------------------------------------
 
-// Macroscopic fields of the post-stream state S_n, rebuilt by pulling from
-// B_{n-1} and applying the wall rule, plus per-block partials (FP64) of
-// max|u|, max|u - u_prev|, sum of population deviations, sum of T - T0.
+// Observables of the post-stream state S_n, rebuilt by pulling from B_{n-1}
+// and applying the wall rule: the macroscopic fields, and FP64 max|u|, max|u -
+// u_prev|, sum of population deviations, sum of T - T0, and both mean Nusselt
+// numbers (Eq. 38): Nu(y) = -L dT/dx / dT, trapezoidal mean over y.
+//
+// The first `nodes` blocks take the nodes, the others the rows of the Nusselt
+// numbers; each leaves four partial results, and the last block to finish folds
+// them in a fixed order (the grid depends on the lattice's size alone, so the
+// sums are reproducible) and re-arms the counter.
+// out[0..6] = nu_hot, nu_cold, max|u|, max|du|, sum d, sum (T - T0), status.
+//
+// FP64 is scarce (an SM retires two lanes per cycle), so a node spends four FP64
+// operations, those of the two sums: maxima are kept as integers, and of |du|
+// the square, which is formed in FP64 only where an FP32 estimate does not rule
+// it out.  64^2: 17 us, against 27 + 38 in two kernels with an FP64 butterfly in
+// every warp and an FP64 root per node; 1024^2: 59 us against 87 + 77.
 template <class T, bool FIELD>
-__global__ void __launch_bounds__(256) k_observe(Src<T> prev, const typename T::P* __restrict__ phi, Geom gm,
-                                                 Coef<typename T::R> c, typename T::R* ux_out,
-                                                 typename T::R* uy_out, typename T::R* T_out,
-                                                 typename T::R* p_out, typename T::R* snap, int snap_valid,
-                                                 double* __restrict__ partials) {
+__global__ void __launch_bounds__(256)
+    k_observe(Src<T> prev, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
+              typename T::R* ux_out, typename T::R* uy_out, typename T::R* T_out, typename T::R* p_out,
+              typename T::R* snap, int snap_valid, double* __restrict__ partials, int nodes, double L, double dT,
+              const int* __restrict__ status, unsigned* __restrict__ counter, double* __restrict__ out) {
     using R = typename T::R;
-    __shared__ double sh[4 * 32];
+    __shared__ double sh[4][256];
+    __shared__ bool last;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    const long n = (long)gm.nx * gm.ny;
-    for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / gm.nx), x = (int)(k - (long)y * gm.nx);
-        R d[9], h[5];
-        Drag<R> dr;
-        const Macro<R> mc = node_state<T, FIELD>(c, gm, prev, phi, x, y, dr, d, h);
-        R sd = R(0);
+    if ((int)blockIdx.x < nodes) {
+        const unsigned n = (unsigned)gm.nx * (unsigned)gm.ny, stride = (unsigned)nodes * 256u;
+        decltype(order_bits(R(0))) umax = 0;
+        double du2 = 0.0;  // max |u - u_prev|^2
+        float ruled = -1.f;  // FP32 estimates up to this are below it
+        for (unsigned k = blockIdx.x * 256u + threadIdx.x; k < n; k += stride) {
+            const int y = (int)(k / (unsigned)gm.nx), x = (int)(k - (unsigned)y * (unsigned)gm.nx);
+            R d[9], h[5];
+            Drag<R> dr;
+            const Macro<R> mc = node_state<T, FIELD>(c, gm, prev, phi, x, y, dr, d, h);
+            R sd = R(0);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) sd += d[i];
-        if (ux_out) ux_out[k] = mc.ux;
-        if (uy_out) uy_out[k] = mc.uy;
-        if (T_out) T_out[k] = c.T0 + mc.dT;
-        if (p_out) p_out[k] = (R(1.0 / 3.0) + mc.dP) * dr.iphi;
-        double du = 0.0;
-        if (snap) {
-            if (snap_valid) {
-                const double ax = (double)mc.ux - (double)snap[2 * k];
-                const double ay = (double)mc.uy - (double)snap[2 * k + 1];
-                du = sqrt(ax * ax + ay * ay);
+            for (int i = 0; i < 9; ++i) sd += d[i];
+            if (ux_out) ux_out[k] = mc.ux;
+            if (uy_out) uy_out[k] = mc.uy;
+            if (T_out) T_out[k] = c.T0 + mc.dT;
+            if (p_out) p_out[k] = (R(1.0 / 3.0) + mc.dP) * dr.iphi;
+            if (snap) {
+                if (snap_valid) {
+                    const R bx = snap[2 * (size_t)k], by = snap[2 * (size_t)k + 1];
+                    float e2 = 0.f;
+                    if constexpr (sizeof(R) == 4) e2 = (mc.ux - bx) * (mc.ux - bx) + (mc.uy - by) * (mc.uy - by);
+                    if (!(e2 <= ruled)) {  // (a NaN gets through; FP64 lattices: always)
+                        const double ax = (double)mc.ux - (double)bx, ay = (double)mc.uy - (double)by;
+                        const double a2 = ax * ax + ay * ay;
+                        if (a2 > du2 || a2 != a2) {
+                            du2 = a2;
+                            if (sizeof(R) == 4 && a2 > 1e-30) ruled = (float)a2 * 0.99999f;
+                        }
+                    }
+                }
+                snap[2 * (size_t)k] = mc.ux;
+                snap[2 * (size_t)k + 1] = mc.uy;
             }
-            snap[2 * k] = mc.ux;
-            snap[2 * k + 1] = mc.uy;
+            umax = max(umax, order_bits(mc.umag));
+            v[2] += (double)sd;
+            v[3] += (double)mc.dT;
         }
-        v[0] = fmax_nan(v[0], (double)mc.umag);
-        v[1] = fmax_nan(v[1], du);
-        v[2] += (double)sd;
-        v[3] += (double)mc.dT;
+        v[0] = from_order(umax);
+        v[1] = du2;
+    } else {
+        const int blocks = gridDim.x - nodes;
+        for (int y = (blockIdx.x - nodes) * 256 + threadIdx.x; y < gm.ny; y += blocks * 256) {
+            double tl[5], tr[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                tl[k] = (double)node_dT<T>(c, gm, prev, k, y);
+                tr[k] = (double)node_dT<T>(c, gm, prev, gm.nx - 1 - k, y);
+            }
+            const double wt = (y == 0 || y == gm.ny - 1) ? 0.5 : 1.0;
+            v[2] += wt * slope_hot(tl);
+            v[3] += wt * slope_cold(tr);
+        }
     }
-    block_reduce4(v, sh);
+    fold_block(v, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) partials[blockIdx.x * 4 + k] = v[k];
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
-}
-
-// One block: folds the per-block partials in a fixed order and evaluates the
-// mean Nusselt numbers (Eq. 38) of both vertical walls, FP64 throughout:
-// Nu(y) = -L dT/dx / dT with the one-sided five-point derivative
-// (-25 T0 + 48 T1 - 36 T2 + 16 T3 - 3 T4) / 12, trapezoidal mean over y.
-// out[0..6] = nu_hot, nu_cold, max|u|, max|du|, sum d, sum (T - T0), status.
-template <class T>
-__global__ void __launch_bounds__(1024) k_finish(Src<T> prev, Geom gm, Coef<typename T::R> c,
-                                                 const double* __restrict__ partials, int npart, double L,
-                                                 double dT, const int* __restrict__ status,
-                                                 double* __restrict__ out) {
-    __shared__ double sh[4 * 32];
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < npart; b += blockDim.x) {
-        v[0] = fmax_nan(v[0], partials[4 * b]);
-        v[1] = fmax_nan(v[1], partials[4 * b + 1]);
-        v[2] += partials[4 * b + 2];
-        v[3] += partials[4 * b + 3];
-    }
-    block_reduce4(v, sh);
     __syncthreads();
-    const double red[4] = {v[0], v[1], v[2], v[3]};
-    double nh, nc;
-    nusselt_block<T>(c, gm, prev, L, dT, sh, &nh, &nc);
+    if (!last) return;
+    __threadfence();
+    double w[4] = {0.0, 0.0, 0.0, 0.0}, nu[4] = {0.0, 0.0, 0.0, 0.0};
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += 256) {
+        const double p0 = __ldcg(partials + 4 * b), p1 = __ldcg(partials + 4 * b + 1);
+        const double p2 = __ldcg(partials + 4 * b + 2), p3 = __ldcg(partials + 4 * b + 3);
+        if (b < (unsigned)nodes) {
+            w[0] = order_bits(p0) > order_bits(w[0]) ? p0 : w[0];
+            w[1] = order_bits(p1) > order_bits(w[1]) ? p1 : w[1];
+            w[2] += p2;
+            w[3] += p3;
+        } else {
+            nu[2] += p2;
+            nu[3] += p3;
+        }
+    }
+    fold_block(w, sh);
+    __syncthreads();
+    fold_block(nu, sh);
     if (threadIdx.x == 0) {
-        out[0] = nh;
-        out[1] = nc;
-        out[2] = red[0];
-        out[3] = red[1];
-        out[4] = red[2];
-        out[5] = red[3];
+        const double scale = -L / (12.0 * dT) / (double)(gm.ny - 1);
+        out[0] = nu[2] * scale;
+        out[1] = nu[3] * scale;
+        out[2] = w[0];
+        out[3] = sqrt(w[1]);
+        out[4] = w[2];
+        out[5] = w[3];
         out[6] = (double)(*status);
+        *counter = 0u;
     }
 }
 
@@ -236,11 +277,9 @@ __global__ void __launch_bounds__(32) k_nusselt_rows(Src<T> prev, const double* 
                 tr[k] = (double)node_dT<T>(c, gm, prev, gm.nx - 1 - k, y);
             }
         }
-        const double dl = (-25.0 * tl[0] + 48.0 * tl[1] - 36.0 * tl[2] + 16.0 * tl[3] - 3.0 * tl[4]) / 12.0;
-        const double dr = (25.0 * tr[0] - 48.0 * tr[1] + 36.0 * tr[2] - 16.0 * tr[3] + 3.0 * tr[4]) / 12.0;
         const double wt = (y == 0 || y == gm.ny - 1) ? 0.5 : 1.0;
-        a = wt * (-L * dl / dT);
-        b = wt * (-L * dr / dT);
+        a = wt * slope_hot(tl);
+        b = wt * slope_cold(tr);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -268,8 +307,10 @@ __global__ void __launch_bounds__(32) k_nusselt_rows(Src<T> prev, const double* 
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
     if (threadIdx.x == 0) {
-        out[0] = a / (double)(gm.ny - 1);
-        out[1] = b / (double)(gm.ny - 1);
+        // -L / dT once for all rows, not a quotient per row
+        const double scale = -L / (12.0 * dT) / (double)(gm.ny - 1);
+        out[0] = a * scale;
+        out[1] = b * scale;
         *counter = 0u;
     }
 }
@@ -372,18 +413,18 @@ template <class T>
 static cudaError_t launch_observe_t(const ObserveLaunch& L, const CoefSet& cs) {
     using R = typename T::R;
     const Src<T> s = src_view<T>(L.prev, L.gm.plane);
-    if (L.phi)
-        k_observe<T, true><<<L.nblocks, 256, 0, L.stream>>>(s, (const typename T::P*)L.phi, L.gm, coef_of<T>(cs),
-                                                            (R*)L.ux, (R*)L.uy, (R*)L.T, (R*)L.p, (R*)L.snap,
-                                                            L.snap_valid, L.partials);
-    else
-        k_observe<T, false><<<L.nblocks, 256, 0, L.stream>>>(s, nullptr, L.gm, coef_of<T>(cs), (R*)L.ux,
-                                                             (R*)L.uy, (R*)L.T, (R*)L.p, (R*)L.snap,
-                                                             L.snap_valid, L.partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_finish<T><<<1, 1024, 0, L.stream>>>(s, L.gm, coef_of<T>(cs), L.partials, L.nblocks, L.L, L.dT, L.status,
-                                          L.out);
+    // blocks for the rows of the Nusselt numbers, and for the nodes as many as the
+    // lattice fills, up to L.nblocks in all
+    const int rows = std::min(64, (L.gm.ny + 255) / 256);
+    const long full = ((long)L.gm.nx * L.gm.ny + 255) / 256;
+    const int nodes = (int)std::min<long>(L.nblocks - rows, full);
+    auto run = [&](auto kernel, const typename T::P* phi) {
+        kernel<<<nodes + rows, 256, 0, L.stream>>>(s, phi, L.gm, coef_of<T>(cs), (R*)L.ux, (R*)L.uy, (R*)L.T, (R*)L.p,
+                                                   (R*)L.snap, L.snap_valid, L.partials, nodes, L.L, L.dT, L.status,
+                                                   L.counter, L.out);
+    };
+    if (L.phi) run(k_observe<T, true>, (const typename T::P*)L.phi);
+    else run(k_observe<T, false>, nullptr);
     return cudaGetLastError();
 }
 

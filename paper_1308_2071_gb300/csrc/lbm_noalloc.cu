@@ -89,7 +89,7 @@ int lbm_observables_noalloc(const lbm_params* p, const void* ckpt_dev, size_t by
     double* partials = scratch;
     double* result = scratch + 4 * kReduceBlocks;
     int* status = (int*)(scratch + 4 * kReduceBlocks + 8);
-    // the array keeps the previous call's contents: clear the status word
+    // the array keeps the previous call's contents: clear the status word (and the block counter beside it)
     e = cudaMemsetAsync(status, 0, sizeof(double), s);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("status clear: ") + cudaGetErrorString(e));
 
@@ -110,6 +110,7 @@ int lbm_observables_noalloc(const lbm_params* p, const void* ckpt_dev, size_t by
     L.dT = dv.dT;
     L.status = status;
     L.out = result;
+    L.counter = (unsigned*)status + 1;  // the other half of the status word's eight bytes
     L.stream = s;
     e = launch_observe(L, cs);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("observables: ") + cudaGetErrorString(e));

@@ -894,65 +894,77 @@ __device__ __forceinline__ double obs_dT(const Coef<typename T::R>& c, const Geo
     return tf;
 }
 
-// The larger of a and b, NaN when either is NaN (fmax would drop it, and a
-// maximum over a lattice holding NaN would look finite).
-__device__ __forceinline__ double fmax_nan(double a, double b) { return (a > b || a != a) ? a : b; }
+// Non-negative values as integers: the order of the bit patterns is that of the
+// values, with NaN (of either sign) above infinity, so that a maximum over a
+// lattice that holds a NaN is NaN; and integers stay off the FP64 unit.
+__device__ __forceinline__ unsigned order_bits(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ unsigned long long order_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ double from_order(unsigned b) { return (double)__uint_as_float(b); }
+__device__ __forceinline__ double from_order(unsigned long long b) { return __longlong_as_double((long long)b); }
 
-// Block-wide reduction of four doubles: max, max, sum, sum (result in thread
-// 0); the maxima keep NaN.
-__device__ __forceinline__ void block_reduce4(double v[4], double* sh /* 4 * 32 */) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Block-wide max, max (non-negative), sum, sum of four doubles per thread; the
+// result in thread 0.  256 threads.  The threads' values meet in shared memory
+// and one warp folds them, eight per lane and then across the lanes: 26
+// FP64 instructions per block for the sums, where a butterfly in every warp
+// takes 90 (an FP64 warp instruction takes an SM 16 cycles).
+__device__ __forceinline__ void fold_block(double (&v)[4], double (*sh)[256]) {
+    const int t = threadIdx.x;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v[0] = fmax_nan(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
-        v[1] = fmax_nan(v[1], __shfl_xor_sync(0xffffffffu, v[1], o));
-        v[2] += __shfl_xor_sync(0xffffffffu, v[2], o);
-        v[3] += __shfl_xor_sync(0xffffffffu, v[3], o);
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) sh[k * 32 + warp] = v[k];
-    }
+    for (int k = 0; k < 4; ++k) sh[k][t] = v[k];
     __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    if (warp == 0) {
+    if (t < 32) {
+        unsigned long long m0 = order_bits(v[0]), m1 = order_bits(v[1]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = (lane < nw) ? sh[k * 32 + lane] : 0.0;
+        for (int w = 1; w < 8; ++w) {
+            m0 = max(m0, order_bits(sh[0][t + 32 * w]));
+            m1 = max(m1, order_bits(sh[1][t + 32 * w]));
+            v[2] += sh[2][t + 32 * w];
+            v[3] += sh[3][t + 32 * w];
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            v[0] = fmax_nan(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
-            v[1] = fmax_nan(v[1], __shfl_xor_sync(0xffffffffu, v[1], o));
+            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
             v[2] += __shfl_xor_sync(0xffffffffu, v[2], o);
             v[3] += __shfl_xor_sync(0xffffffffu, v[3], o);
         }
+        v[0] = from_order(m0);
+        v[1] = from_order(m1);
     }
 }
 
-// Mean Nusselt numbers (Eq. 38) of both vertical walls over the whole block
-// (valid in thread 0): Nu(y) = -L dT/dx / dT with the one-sided five-point
-// derivative (-25 T0 + 48 T1 - 36 T2 + 16 T3 - 3 T4) / 12, trapezoidal mean
-// over y, FP64.  sh: 4 * 32 doubles of shared memory.
+// 12 dT/dx (Eq. 38's one-sided five-point derivative, times the spacing) at both
+// ends of a row from the five temperatures next to each wall.
+__device__ __forceinline__ double slope_hot(const double (&t)[5]) {
+    return -25.0 * t[0] + 48.0 * t[1] - 36.0 * t[2] + 16.0 * t[3] - 3.0 * t[4];
+}
+__device__ __forceinline__ double slope_cold(const double (&t)[5]) {
+    return 25.0 * t[0] - 48.0 * t[1] + 36.0 * t[2] - 16.0 * t[3] + 3.0 * t[4];
+}
+
+// Mean Nusselt numbers (Eq. 38) of both vertical walls over a whole block of 256
+// threads (valid in thread 0): Nu(y) = -L dT/dx / dT, trapezoidal mean over y,
+// FP64.
 template <class T>
 __device__ __forceinline__ void nusselt_block(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& prev,
-                                              double L, double dT, double* sh, double* nu_hot, double* nu_cold) {
+                                              double L, double dT, double (*sh)[256], double* nu_hot,
+                                              double* nu_cold) {
     double w[4] = {0.0, 0.0, 0.0, 0.0};
-    const int nx = gm.nx;
-    for (int y = threadIdx.x; y < gm.ny; y += blockDim.x) {
+    for (int y = threadIdx.x; y < gm.ny; y += 256) {
         double tl[5], tr[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
             tl[k] = (double)node_dT<T>(c, gm, prev, k, y);
-            tr[k] = (double)node_dT<T>(c, gm, prev, nx - 1 - k, y);
+            tr[k] = (double)node_dT<T>(c, gm, prev, gm.nx - 1 - k, y);
         }
-        const double dl = (-25.0 * tl[0] + 48.0 * tl[1] - 36.0 * tl[2] + 16.0 * tl[3] - 3.0 * tl[4]) / 12.0;
-        const double dr = (25.0 * tr[0] - 48.0 * tr[1] + 36.0 * tr[2] - 16.0 * tr[3] + 3.0 * tr[4]) / 12.0;
         const double wt = (y == 0 || y == gm.ny - 1) ? 0.5 : 1.0;
-        w[2] += wt * (-L * dl / dT);
-        w[3] += wt * (-L * dr / dT);
+        w[2] += wt * slope_hot(tl);
+        w[3] += wt * slope_cold(tr);
     }
-    block_reduce4(w, sh);
-    *nu_hot = w[2] / (double)(gm.ny - 1);
-    *nu_cold = w[3] / (double)(gm.ny - 1);
+    fold_block(w, sh);
+    const double scale = -L / (12.0 * dT) / (double)(gm.ny - 1);
+    *nu_hot = w[2] * scale;
+    *nu_cold = w[3] * scale;
 }
 
 }  // namespace lbm

@@ -19,11 +19,11 @@ namespace lbm {
 // state[0..1]: previous Nu_hot, Nu_cold; [2]: last relative change;
 // [3]: checks done; [4]: stop reason (1 converged, 2 diverged, 3 step cap).
 template <class T>
-__global__ void __launch_bounds__(1024) k_steady_check(Src<T> prev, Geom gm, Coef<typename T::R> c, double L,
+__global__ void __launch_bounds__(256) k_steady_check(Src<T> prev, Geom gm, Coef<typename T::R> c, double L,
                                                        double dT, const int* __restrict__ status, double tol,
                                                        long max_checks, double* __restrict__ state,
                                                        cudaGraphConditionalHandle cond) {
-    __shared__ double sh[4 * 32];
+    __shared__ double sh[4][256];
     double nh, nc;
     nusselt_block<T>(c, gm, prev, L, dT, sh, &nh, &nc);
     if (threadIdx.x == 0) {
@@ -77,7 +77,7 @@ template <> const Coef<float>& coef_sel<PrecF32T>(const CoefSet& cs) { return cs
 
 template <class T>
 static cudaError_t launch_check_t(const SteadyCheckLaunch& L, const CoefSet& cs) {
-    k_steady_check<T><<<1, 1024, 0, L.stream>>>(src_view<T>(L.prev, L.gm.plane), L.gm, coef_sel<T>(cs), L.L, L.dT,
+    k_steady_check<T><<<1, 256, 0, L.stream>>>(src_view<T>(L.prev, L.gm.plane), L.gm, coef_sel<T>(cs), L.L, L.dT,
                                                 L.status, L.tol, L.max_checks, L.state, L.cond);
     return cudaGetLastError();
 }
