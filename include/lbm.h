@@ -201,9 +201,9 @@ int lbm_step_nusselt(lbm_handle h, long nsteps, double* out);
 
 /* Discrete adjoint (no counterpart in the paper, which has no gradient).
  * Resets the handle to its initial state, runs nsteps steps forward keeping
- * one lattice every ckpt_every steps, evaluates J = mean Nu of the hot wall
- * (Eq. 38) at t = nsteps, then sweeps backwards, recomputing each segment of
- * ckpt_every states from its checkpoint, and writes dJ/dphi for every cell
+ * one lattice at least every ckpt_every steps, evaluates J = mean Nu of the hot wall
+ * (Eq. 38) at t = nsteps, then sweeps backwards, recomputing each segment from
+ * its checkpoint, and writes dJ/dphi for every cell
  * (ny*nx dense device values, double for LBM_F64, float for the FP32
  * variants) to dJdphi_dev; *J (host, may be NULL) receives J.  The porosity
  * enters through the per-cell Ergun drag (Eq. 4-5) and the equilibria (Eq.
@@ -212,8 +212,9 @@ int lbm_step_nusselt(lbm_handle h, long nsteps, double* out);
  * The recomputation of each segment runs on a stream of its own, beside the
  * reverse sweep of the segment after it.  The handle ends at t = nsteps.
  * Needs use_phi_field = 1, LBM_F64, LBM_F32 or LBM_F32_FRAMED, first-order
- * adiabatic walls.  Allocates (nsteps/ckpt_every + 2 ckpt_every + 1)
- * lattices of temporary device memory for the call.  Synchronises.
+ * adiabatic walls.  Allocates nsteps/K + 2 K + 1 lattices of temporary device
+ * memory for the call, K = min(ckpt_every, sqrt(nsteps / 2)) (a longer interval
+ * would take more); the gradient's bits do not depend on it.  Synchronises.
  * Errors: LBM_ERR_STATE (no porosity field), LBM_ERR_ARG, LBM_ERR_CUDA. */
 int lbm_adjoint_step(lbm_handle h, long nsteps, long ckpt_every, double* J, void* dJdphi_dev);
 

@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lbm_adjoint.cuh"
@@ -22,6 +23,8 @@
 using namespace lbm;
 
 namespace lbm {
+
+constexpr int kAdjThreads = 128, kAdjBlocks = 5;
 
 // dJ/dS_N as the initial adjoint state: J depends on T at the columns 1..4
 // next to the hot wall (the wall column is the imposed T_h); on first-order
@@ -42,140 +45,222 @@ __global__ void k_adj_seed(R* __restrict__ M, Geom gm, double L, double dT) {
     }
 }
 
-template <class R>
-__device__ __forceinline__ void gather_adjoint(const R* __restrict__ M, const Geom& gm, int x, int y, R (&lf)[9],
-                                               R (&lh)[5]) {
+// Element at a uniform base and a thread's byte offset: one register serves every
+// plane and neighbour, and the planes' bases stay in uniform registers (with an
+// index per access, half of the kernel's instructions were addresses).  The
+// offset fits 32 bits: a lattice of 2^32 bytes per plane takes over 300 GB here.
+template <class S> __device__ __forceinline__ S* at(S* base, unsigned bytes) {
+    if constexpr (std::is_const<S>::value) return (S*)((const char*)base + bytes);
+    else return (S*)((char*)base + bytes);
+}
+
+// lambda and mu of node (x, y): the adjoint of what it sent along each e_i.
+// Plain loads, not the read-only path: a launch may start while the one that
+// wrote these values is still running (it reads them after its wait).
+// EDGE: next to or on a wall, where neighbours may lie outside.
+template <class R, bool EDGE>
+__device__ __forceinline__ void gather_adjoint(const R* M, const Geom& gm, int x, int y, R (&l)[9], R (&m)[5]) {
+    const unsigned off = (unsigned)(y * gm.pitch + x) * (unsigned)sizeof(R);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const int xs = x + ex9(i), ys = y + ey9(i);
-        const bool in = xs >= 0 && xs < gm.nx && ys >= 0 && ys < gm.ny;
-        lf[i] = in ? M[i * gm.plane + ys * gm.pitch + xs] : R(0);
+    for (int q = 0; q < NPOP; ++q) {
+        const int i = q < 9 ? q : q - 9, xs = x + ex9(i), ys = y + ey9(i);
+        const bool in = !EDGE || (xs >= 0 && xs < gm.nx && ys >= 0 && ys < gm.ny);
+        const R v = in ? __ldcg(at(M + (q * gm.plane + ey9(i) * gm.pitch + ex9(i)), off)) : R(0);
+        if (q < 9) l[q] = v;
+        else m[q - 9] = v;
+    }
+}
+
+// What the transpose needs of the populations pulled into a fluid node (a and b
+// only next to a wall).
+template <class T>
+__device__ __forceinline__ void tape_at(const Coef<typename T::R>& c, const Src<T>& src, const Geom& gm,
+                                        const typename T::P* __restrict__ phi, int off, Tape<typename T::R>& t) {
+    using R = typename T::R;
+    R d[9], h[5];
+    d[0] = R(0);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        const int o = off - ey9(i) * gm.pitch - ex9(i);
+        d[i] = in_plane(gm, o) ? Conv<typename T::SF, R, T::cg>::ld(src.f + i * gm.plane + o) : R(0);
     }
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-        const int xs = x + ex9(j), ys = y + ey9(j);
-        const bool in = xs >= 0 && xs < gm.nx && ys >= 0 && ys < gm.ny;
-        lh[j] = in ? M[(9 + j) * gm.plane + ys * gm.pitch + xs] : R(0);
+        const int o = off - ey9(j) * gm.pitch - ex9(j);
+        h[j] = in_plane(gm, o) ? Conv<typename T::SG, R, T::cg>::ld(src.g + j * gm.plane + o) : R(0);
     }
+    const R F = op::mul(core_frame_in<T>(c.k, src, gm, off, h), c.k.fu);
+    tape_node<R, Framed<T>::value>(c.k, (R)phi[off], sums_of(d, h), F, t);
 }
 
-// The populations pulled into node off, as deviations from the rest state:
-// with framed storage the thermal values are re-expressed relative to T0
-// (the frame is an exact change of variables of the stored values, so the
-// adjoint of the step is the one of the plain deviations).
-template <class T>
-__device__ __forceinline__ void pull_rest(const Coef<typename T::R>& c, const Src<T>& src, const Geom& gm, int off,
-                                          typename T::R (&d)[9], typename T::R (&h)[5]) {
-    pull<T>(src, gm, off, d, h);
-    if constexpr (Framed<T>::value) {
-        const typename T::R F = frame_in<T>(c, src, gm, off, h);
-        h[0] += c.wt0 * F;
-#pragma unroll
-        for (int j = 1; j < 5; ++j) h[j] += c.wt1 * F;
-    }
-}
-
-__device__ __forceinline__ bool wall_is_dirichlet(const Geom& gm, Normal nr) {
-    return gm.thermal_bc == 1 || nr.dx != 0;
-}
-
-template <class R>
-__device__ __forceinline__ R wall_dT(const Coef<R>& c, const Geom& gm, int x) {
-    return gm.thermal_bc == 1 ? c.dTc : (x == 0 ? c.dTh : c.dTc);
-}
-
-// Reverse of one node for one step: from M^(k+1) and the forward input B_k
-// to M^(k) at (x, y), adding this step's porosity sensitivity to gphi.
-// RING = false: (x, y) is at least two nodes from every wall, so it is a
-// fluid node and no wall node extrapolates from it.
-template <class T, bool RING>
-__device__ __forceinline__ void adjoint_node(const Src<T>& state, const typename T::R* __restrict__ Mnext,
-                                             typename T::R* __restrict__ Mcur, const typename T::P* __restrict__ phi,
-                                             double* __restrict__ gphi, const Geom& gm, const Coef<typename T::R>& c,
-                                             int x, int y) {
+// Two nodes side by side (x0 even): values whose two nodes start at an even x
+// come as pairs.
+template <class T> struct PairAt {
     using R = typename T::R;
-    const int off = y * gm.pitch + x;
-    const long k = (long)y * gm.nx + x;
-    const Normal nr = normal_of(gm, x, y);
-    R lf[9], lh[5];
-    if (RING && (nr.dx != 0 || nr.dy != 0)) {
-        // wall node: it reads no pulled populations of its own; its porosity
-        // sensitivity is computed here, its inner neighbour's by that node
+    // plane p's values that e_i carries into the pair at off
+    static __device__ __forceinline__ float2 state(const float* p, const Geom& gm, int off, int ex, int ey) {
+        const int d = -ey * gm.pitch - ex;
+        const unsigned b = 4u * (unsigned)off;
+        if (ex == 0)
+            return in_plane(gm, off + d, 2) ? Conv2<float, float, T::cg>::ld(at(p + d, b)) : make_float2(0.f, 0.f);
+        return make_float2(in_plane(gm, off + d) ? Conv<float, float, T::cg>::ld(at(p + d, b)) : 0.f,
+                           in_plane(gm, off + d + 1) ? Conv<float, float, T::cg>::ld(at(p + d, b) + 1) : 0.f);
+    }
+    static __device__ __forceinline__ void tape(const Coef<float>& c, const Src<T>& src, const Geom& gm,
+                                                const float* __restrict__ phi, int off, Tape<F2>& t) {
+        float h0[5], h1[5], F0, F1;
+        F2 d[9], h[5];
+        d[0] = F2(0.f);
 #pragma unroll
-        for (int q = 0; q < NPOP; ++q) Mcur[q * gm.plane + off] = R(0);
-        gather_adjoint<R>(Mnext, gm, x, y, lf, lh);
-        const int xf = x + nr.dx, yf = y + nr.dy, offf = yf * gm.pitch + xf;
-        R df[9], hf[5];
-        pull_rest<T>(c, state, gm, offf, df, hf);
-        Tape<R> tf;
-        tape_node<R>(c, (R)phi[offf], df, hf, tf);
-        R dfb[9] = {R(0)}, hfb[5] = {R(0)}, pfb = R(0);
-        const R pb = wall_node_adjoint<R>(c, tf, (R)phi[off], wall_is_dirichlet(gm, nr), wall_dT<R>(c, gm, x), lf, lh,
-                                          dfb, hfb, pfb);
-        gphi[k] += (double)pb;
+        for (int i = 1; i < 9; ++i)
+            d[i] = F2(state(src.f + i * gm.plane, gm, off, ex9(i), ey9(i)));
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const float2 v = state(src.g + j * gm.plane, gm, off, ex9(j), ey9(j));
+            h0[j] = v.x;
+            h1[j] = v.y;
+        }
+        core_frame_in_x2<T>(c.k, src, gm, off, h0, h1, F0, F1);
+#pragma unroll
+        for (int j = 0; j < 5; ++j) h[j] = F2(h0[j], h1[j]);
+        const float2 ph = __ldg((const float2*)at(phi, 4u * (unsigned)off));
+        tape_node<F2, Framed<T>::value>(c.k, F2(ph), sums_of(d, h), op::mul(c.k.fu, F2(F0, F1)), t);
+    }
+    static __device__ __forceinline__ void gather(const float* M, const Geom& gm, int off, F2 (&l)[9], F2 (&m)[5]) {
+#pragma unroll
+        for (int q = 0; q < NPOP; ++q) {
+            const int i = q < 9 ? q : q - 9;
+            const float* p = at(M + (q * gm.plane + ey9(i) * gm.pitch + ex9(i)), 4u * (unsigned)off);
+            const F2 v = ex9(i) == 0 ? F2(__ldca((const float2*)p)) : F2(__ldca(p), __ldca(p + 1));
+            if (q < 9) l[q] = v;
+            else m[q - 9] = v;
+        }
+    }
+};
+
+// n / d for n < 2^31 by a multiplication (d >= 2: m = ceil(2^(31 + l) / d), l = ceil(log2 d))
+struct Divider {
+    unsigned m = 0, s = 0;
+    explicit Divider(unsigned d) {
+        if (d < 2) return;
+        unsigned l = 1;
+        while ((1ull << l) < d) ++l;
+        m = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
+        s = l - 1;
+    }
+    __device__ __forceinline__ int quotient(unsigned n) const { return (int)(m ? __umulhi(n, m) >> s : n); }
+};
+
+// Reverse of one step at the interior nodes, two or more from every wall, and in
+// the first `edge` blocks (their nodes take longer) at the fluid nodes next to a
+// wall together with the wall nodes that extrapolate from them: M^(k) from
+// M^(k+1) and the forward input B_k, and this step's porosity sensitivity added
+// to gphi.  M at the wall nodes stays 0: they read no pulled populations of
+// their own.
+//
+// The state and the tape need nothing of the previous reverse step, so a launch
+// starts early, as a programmatic dependent, and waits only then (late start:
+// 10.8 ms instead of 10.0 for the call below).
+//
+// Everything but the forward states stays in L2; a step moves 72 MB through it
+// at 512^2 and is bound by that latency and by issue slots (540 instructions per
+// pair, 202 of them arithmetic; 1.35 waves of 20 warps per SM).  512^2 FP32, us
+// per reverse step alone: 7.6; 8.3 with an index per access, and 23.4 for the
+// direct formulas in one kernel for the interior and one for the ring of nodes
+// near the walls on a stream of its own.  The gradient of 600 steps: 19.8 -> 10.2 ms.
+template <class T>
+__global__ void __launch_bounds__(kAdjThreads, sizeof(typename T::R) == 4 ? kAdjBlocks : 2)
+    k_adjoint(Src<T> state, const typename T::R* Mnext, typename T::R* Mcur, const typename T::P* __restrict__ phi,
+              double* gphi, Geom gm, Coef<typename T::R> c, int edge, Divider rows_of) {
+    using R = typename T::R;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if ((int)blockIdx.x < edge) {
+        const int j = blockIdx.x * kAdjThreads + threadIdx.x, rows = 2 * (gm.nx - 2);
+        int x = 0, y = 0;
+        const bool in = j < rows + 2 * (gm.ny - 4);
+        Tape<R> t;
+        if (in) {
+            if (j < rows) {
+                x = 1 + (j >> 1);
+                y = j & 1 ? gm.ny - 2 : 1;
+            } else {
+                x = j & 1 ? gm.nx - 2 : 1;
+                y = 2 + ((j - rows) >> 1);
+            }
+            tape_at<T>(c, state, gm, phi, y * gm.pitch + x, t);
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (!in) return;
+        const int off = y * gm.pitch + x;
+        R l[9], m[5];
+        gather_adjoint<R, true>(Mnext, gm, x, y, l, m);
+        Seeds<R> b = {};
+        own_seeds(c.k, l[0], sums_of(l, m), b);
+        const int sx = x == 1 ? -1 : x == gm.nx - 2 ? 1 : 0, sy = y == 1 ? -1 : y == gm.ny - 2 ? 1 : 0;
+#pragma unroll 1
+        for (int w = 0; w < 3; ++w) {  // the wall nodes beside, below or above, and across the corner
+            if ((w != 1 && sx == 0) || (w != 0 && sy == 0)) continue;
+            const int xb = w == 1 ? x : x + sx, yb = w == 0 ? y : y + sy;
+            R lb[9], mb[5];
+            gather_adjoint<R, true>(Mnext, gm, xb, yb, lb, mb);
+            const bool dirichlet = gm.thermal_bc == 1 || w != 1;
+            const R dTw = gm.thermal_bc == 0 && xb == 0 ? c.k.dTh : c.k.dTc;
+            const R pb = wall_seeds<R>(c.k, t, (R)phi[yb * gm.pitch + xb], dirichlet, dTw, lb[0], mb[0],
+                                       sums_of(lb, mb), b);
+            gphi[(long)yb * gm.nx + xb] += (double)pb;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) l[i] = op::add(l[i], lb[i]);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) m[i] = op::add(m[i], mb[i]);
+        }
+        const R pb = node_adjoint<R, true>(c.k, t, b, sums_of(l, m), l, m);
+#pragma unroll
+        for (int q = 0; q < NPOP; ++q) Mcur[q * gm.plane + off] = q < 9 ? l[q] : m[q - 9];
+        gphi[(long)y * gm.nx + x] += (double)pb;
         return;
     }
-    gather_adjoint<R>(Mnext, gm, x, y, lf, lh);
-    R d[9], h[5];
-    pull_rest<T>(c, state, gm, off, d, h);
-    Tape<R> t;
-    tape_node<R>(c, (R)phi[off], d, h, t);
-    R db[9] = {R(0)}, hb[5] = {R(0)}, pb = R(0);
-    fluid_node_adjoint<R>(c, t, lf, lh, db, hb, pb);
-    // wall nodes b = x - n whose inward normal n points at this node
-    if (RING)
-    for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-            if (dx == 0 && dy == 0) continue;
-            const int xb = x - dx, yb = y - dy;
-            const Normal nb = normal_of(gm, xb, yb);
-            if (nb.dx != dx || nb.dy != dy) continue;
-            R lfb[9], lhb[5];
-            gather_adjoint<R>(Mnext, gm, xb, yb, lfb, lhb);
-            (void)wall_node_adjoint<R>(c, t, (R)phi[yb * gm.pitch + xb], wall_is_dirichlet(gm, nb),
-                                       wall_dT<R>(c, gm, xb), lfb, lhb, db, hb, pb);
-        }
+    const int n = (blockIdx.x - edge) * kAdjThreads + threadIdx.x;
+    if constexpr (sizeof(R) == 4) {  // FP32: two nodes per thread
+        const int w = (gm.nx - 3) / 2, yi = rows_of.quotient(n), x = 2 + 2 * (n - yi * w), y = 2 + yi, off = y * gm.pitch + x;
+        const bool in = yi < gm.ny - 4;
+        Tape<F2> t;
+        if (in) PairAt<T>::tape(c, state, gm, phi, off, t);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (!in) return;
+        double* g = gphi + ((long)y * gm.nx + x);
+        const bool two = x + 1 < gm.nx - 2;  // else the second node is next to the wall
+        F2 l[9], m[5];
+        PairAt<T>::gather(Mnext, gm, off, l, m);
+        const double g0 = __ldcg(g), g1 = __ldcg(g + 1);
+        const Sums<F2> s = sums_of(l, m);
+        Seeds<F2> b;
+        own_seeds(c.k, l[0], s, b);
+        const F2 pb = node_adjoint<F2, false>(c.k, t, b, s, l, m);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) Mcur[i * gm.plane + off] = db[i];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) Mcur[(9 + j) * gm.plane + off] = hb[j];
-    gphi[k] += (double)pb;
-}
-
-// One reverse step over the interior nodes (two or more nodes from every
-// wall), grid-stride over a grid sized to the resident capacity.
-template <class T>
-__global__ void __launch_bounds__(256, sizeof(typename T::R) == 4 ? 4 : 1)
-    k_adjoint(Src<T> state, const typename T::R* __restrict__ Mnext, typename T::R* __restrict__ Mcur,
-              const typename T::P* __restrict__ phi, double* __restrict__ gphi, Geom gm, Coef<typename T::R> c) {
-    const int w = gm.nx - 4;
-    const long n = (long)w * (gm.ny - 4);
-    for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
-        const int yi = (int)(k / w);
-        adjoint_node<T, false>(state, Mnext, Mcur, phi, gphi, gm, c, 2 + (int)(k - (long)yi * w), 2 + yi);
-    }
-}
-
-// The same over the ring of nodes within two of a wall (nx, ny >= 5): rows
-// 0, 1, ny-2, ny-1 in full, then columns 0, 1, nx-2, nx-1 of rows 2..ny-3.
-template <class T>
-__global__ void __launch_bounds__(64)
-    k_adjoint_ring(Src<T> state, const typename T::R* __restrict__ Mnext, typename T::R* __restrict__ Mcur,
-                   const typename T::P* __restrict__ phi, double* __restrict__ gphi, Geom gm,
-                   Coef<typename T::R> c) {
-    const long rows = 4L * gm.nx, n = rows + 4L * (gm.ny - 4);
-    for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
-        int x, y;
-        if (k < rows) {
-            const int r = (int)(k / gm.nx);
-            x = (int)(k - (long)r * gm.nx);
-            y = r < 2 ? r : gm.ny - 4 + r;
-        } else {
-            const int j = (int)(k - rows), r = j >> 2, q = j & 3;
-            y = 2 + r;
-            x = q < 2 ? q : gm.nx - 4 + q;
+        for (int q = 0; q < NPOP; ++q) {
+            const F2 v = q < 9 ? l[q] : m[q - 9];
+            R* p = at(Mcur + q * gm.plane, 4u * (unsigned)off);
+            if (two) *(float2*)p = v.v;
+            else *p = v.v.x;
         }
-        adjoint_node<T, true>(state, Mnext, Mcur, phi, gphi, gm, c, x, y);
+        g[0] = g0 + (double)pb.v.x;
+        if (two) g[1] = g1 + (double)pb.v.y;
+    } else {
+        const int w = gm.nx - 4, yi = rows_of.quotient(n), x = 2 + n - yi * w, y = 2 + yi, off = y * gm.pitch + x;
+        const bool in = yi < gm.ny - 4;
+        Tape<R> t;
+        if (in) tape_at<T>(c, state, gm, phi, off, t);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (!in) return;
+        R l[9], m[5];
+        gather_adjoint<R, false>(Mnext, gm, x, y, l, m);
+        const Sums<R> s = sums_of(l, m);
+        Seeds<R> b;
+        own_seeds(c.k, l[0], s, b);
+        const R pb = node_adjoint<R, false>(c.k, t, b, s, l, m);
+#pragma unroll
+        for (int q = 0; q < NPOP; ++q) Mcur[q * gm.plane + off] = q < 9 ? l[q] : m[q - 9];
+        gphi[(long)y * gm.nx + x] += (double)pb;
     }
 }
 
@@ -189,25 +274,7 @@ __global__ void k_adj_out(const double* __restrict__ g, Out* __restrict__ out, l
 
 namespace {
 
-// Second stream for the ring kernel, and the two events that join it with
-// the main stream around every reverse step.
-struct RingStream {
-    cudaStream_t s2 = nullptr;
-    cudaEvent_t main_done = nullptr, ring_done = nullptr;
-    cudaError_t init() {
-        cudaError_t e = cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&main_done, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ring_done, cudaEventDisableTiming);
-        return e;
-    }
-    ~RingStream() {
-        if (ring_done) cudaEventDestroy(ring_done);
-        if (main_done) cudaEventDestroy(main_done);
-        if (s2) cudaStreamDestroy(s2);  // resources go once its work is done
-    }
-};
-
-// Third stream for the recomputation of the next segment, with an event per
+// Second stream for the recomputation of the next segment, with an event per
 // half of the segment storage for "recomputed" and for "read by the reverse
 // sweep" (both recorded once at the start, so the first waits pass).
 struct RecomputeStream {
@@ -246,36 +313,22 @@ cudaError_t adjoint_sweep(const AdjointJob& J) {
     const size_t buf = J.buf_bytes;
     const size_t mbytes = (size_t)gm.plane * NPOP * sizeof(R);
     cudaStream_t s = J.stream;
-    int dev = 0, nsm = 0, per_sm = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (e0 == cudaSuccess) e0 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adjoint<T>, 256, 0);
-    if (e0 != cudaSuccess) return e0;
-    const long inner = (long)(gm.nx - 4) * (gm.ny - 4), ring = 4L * gm.nx + 4L * (gm.ny - 4);
-    // one interior node per thread: the hardware starts the blocks of the
-    // next wave as blocks finish (a grid-stride loop over fewer resident
-    // blocks ran its last pass with a fifth of the threads busy)
-    (void)per_sm;
-    const int nblk = (int)std::max(1L, (inner + 255) / 256);
-    const int nring = (int)std::max(1L, std::min((long)nsm, (ring + 63) / 64));
+    const int wide = sizeof(R) == 4 ? (gm.nx - 3) / 2 : gm.nx - 4;  // threads per interior row
+    const long inner = (long)wide * (gm.ny - 4);
+    const Divider rows_of((unsigned)wide);
+    const long next = 2L * (gm.nx - 2) + 2L * (gm.ny - 4);
+    const int edge = (int)((next + kAdjThreads - 1) / kAdjThreads);
+    const int nblk = edge + (int)((inner + kAdjThreads - 1) / kAdjThreads);
     const int nseg = (N + K - 1) / K;
     R* M[2] = {(R*)J.madj, (R*)J.madj + (size_t)gm.plane * NPOP};
-    cudaError_t e = cudaMemsetAsync(M[0], 0, mbytes, s);
+    cudaError_t e = cudaMemsetAsync(M[0], 0, 2 * mbytes, s);
     if (e != cudaSuccess) return e;
     k_adj_seed<R><<<(gm.ny + 255) / 256, 256, 0, s>>>(M[0], gm, J.L, J.dT);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(J.gphi, 0, sizeof(double) * (size_t)gm.nx * gm.ny, s)) != cudaSuccess) return e;
-    // Within a reverse step the ring and interior nodes are independent (each
-    // writes its own nodes of M^(k) and gphi), so the ring kernel runs on a
-    // second stream beside the interior kernel; the main stream waits for it
-    // before the next step.  The recomputation of a segment needs only its
-    // checkpoint, so it runs on a third stream into the other half of the
-    // segment storage while the main stream reverses the segment after it:
-    // the latency-bound forward steps and reverse steps overlap.
-    RingStream rs;
-    if ((e = rs.init()) != cudaSuccess) return e;
-    auto join = [&]() { return cudaStreamWaitEvent(s, rs.ring_done, 0); };
-    if ((e = cudaEventRecord(rs.ring_done, rs.s2)) != cudaSuccess) return e;  // nothing pending on s2 yet
+    // The recomputation of a segment needs only its checkpoint, so it runs on a
+    // second stream into the other half of the segment storage while the main
+    // stream reverses the segment after it: forward steps and reverse steps overlap.
     RecomputeStream rc;
     if ((e = rc.init(s)) != cudaSuccess) return e;
     CoefSet cs;
@@ -286,7 +339,7 @@ cudaError_t adjoint_sweep(const AdjointJob& J) {
     auto slot_of = [&](int sg, int hf, int m) -> const void* {
         return m == 0 ? (const char*)J.ckpt + (size_t)sg * buf : (const char*)J.seg + hf * half + (size_t)(m - 1) * buf;
     };
-    // recompute segment sg into half hf on the third stream, once the reverse
+    // recompute segment sg into half hf on the second stream, once the reverse
     // sweep that last read that half is done
     auto recompute = [&](int sg, int hf) -> cudaError_t {
         cudaError_t er = cudaStreamWaitEvent(rc.s3, rc.free[hf], 0);
@@ -316,26 +369,25 @@ cudaError_t adjoint_sweep(const AdjointJob& J) {
         if ((e = cudaStreamWaitEvent(s, rc.ready[hf], 0)) != cudaSuccess) break;
         for (int j = j0 + len - 1; j >= j0; --j) {
             const Src<T> st = src_view<T>(slot_of(sg, hf, j - j0), gm.plane);
-            // main_done: everything before this step (previous step, recompute) has finished on s
-            if ((e = cudaEventRecord(rs.main_done, s)) != cudaSuccess) break;
-            if ((e = cudaStreamWaitEvent(rs.s2, rs.main_done, 0)) != cudaSuccess) break;
-            k_adjoint_ring<T><<<nring, 64, 0, rs.s2>>>(st, M[a], M[a ^ 1], (const typename T::P*)J.phi, J.gphi,
-                                                        gm, c);
-            if ((e = cudaGetLastError()) != cudaSuccess) break;
-            if ((e = cudaEventRecord(rs.ring_done, rs.s2)) != cudaSuccess) break;
-            k_adjoint<T><<<nblk, 256, 0, s>>>(st, M[a], M[a ^ 1], (const typename T::P*)J.phi, J.gphi, gm, c);
-            if ((e = cudaGetLastError()) != cudaSuccess) break;
-            if ((e = join()) != cudaSuccess) break;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(nblk);
+            cfg.blockDim = dim3(kAdjThreads);
+            cfg.stream = s;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = j < j0 + len - 1 ? 1 : 0;  // directly behind a reverse step of the same segment
+            e = cudaLaunchKernelEx(&cfg, k_adjoint<T>, st, (const R*)M[a], M[a ^ 1], (const typename T::P*)J.phi,
+                                   J.gphi, gm, c, edge, rows_of);
+            if (e != cudaSuccess) break;
             a ^= 1;
         }
         // the half is free again once this segment's reverse sweep is done
         if (e == cudaSuccess) e = cudaEventRecord(rc.free[hf], s);
     }
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, rc.done(), 0);
-    if (e != cudaSuccess) {
-        (void)join();  // leave no ring work behind the main stream's back
-        return e;
-    }
+    if (e != cudaSuccess) return e;
     const long n = (long)gm.nx * gm.ny;
     if (sizeof(R) == 8) k_adj_out<double><<<kReduceBlocks, 256, 0, s>>>(J.gphi, (double*)J.out, n);
     else k_adj_out<float><<<kReduceBlocks, 256, 0, s>>>(J.gphi, (float*)J.out, n);

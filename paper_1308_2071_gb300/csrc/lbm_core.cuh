@@ -193,6 +193,7 @@ template <class V> __device__ __forceinline__ Sums<V> sums_of(const V (&d)[9], c
 
 template <class V> struct Vel {
     V ux, uy, dux, duy, vm, ngd;  // u, u - j, |v|, minus the fraction of v that the drag takes
+    V S;                          // 1/2 + sqrt(l0^2 + l1 |v|)
     V dTl, dT;                    // T - T0 - F (framed storage; else T - T0) and T - T0
 };
 
@@ -212,9 +213,9 @@ template <class V, bool FR> __device__ __forceinline__ Vel<V> velocity(const Col
     const V vy = op::add(jy, by);
     m.vm = op::root(op::fma(jx, jx, op::fma(vy, vy, op::tiny(V(0)))));
     const V e = op::fma(p.l1, m.vm, p.ec);
-    const V S = op::add(op::root(op::add(V(Scalar<V>(0.25)), e)), V(Scalar<V>(0.5)));
-    const V w = op::fma(p.cc, S, e);
-    m.ngd = op::mul(w, op::minus_inverse(op::add(S, w)));
+    m.S = op::add(op::root(op::add(V(Scalar<V>(0.25)), e)), V(Scalar<V>(0.5)));
+    const V w = op::fma(p.cc, m.S, e);
+    m.ngd = op::mul(w, op::minus_inverse(op::add(m.S, w)));
     m.dux = op::mul(jx, m.ngd);
     m.duy = op::fma(vy, m.ngd, by);
     m.ux = op::add(jx, m.dux);
