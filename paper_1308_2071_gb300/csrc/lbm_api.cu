@@ -545,14 +545,27 @@ int lbm_init(const lbm_params* p, void* stream, lbm_handle* out) {
     // along x, in one-warp blocks on small lattices, which share them out evenly
     // (200^2 2.3 against 2.9 with 64 x 2 threads, 450^2 3.6 / 4.1, 4096^2 the same);
     // FP64 one node per thread on the smallest (64^2 8.4 / 10.5 / 26.7 with one / two
-    // along y / two in blocks of 64 x 2), else two along y (257^2 21.3 / 46)
+    // along y / two in blocks of 64 x 2), else two along y (257^2 21.3 / 46) as long as
+    // its blocks, eight to an SM by their registers, all run at once (a fiftieth to
+    // spare), or in so many waves that the last does not count; one between (us for
+    // two / one: 257^2 21.1 / 23.0, 264^2 34.7 / 25.0, 280^2 36.4 / 25.7, 400^2 57.8 /
+    // 46.7, 512^2 78.7 / 71.9, 800^2 176 / 172, 900^2 222 / 222, 1024^2 276 / 278), from
+    // 350^2 on in blocks of 32 x 4 (against 32 x 1: 320^2 34.8 / 31.6, 400^2 46.7 / 48.7)
     const long nodes = (long)p->nx * p->ny;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        nsm = 0;  // (an error that persists shows at the first allocation)
+    // blocks of two nodes along y, the border's included
+    const long by_two = (p->nx + 31L) / 32 * ((p->ny - 1) / 2) + (p->nx + p->ny) / 16;
+    const bool two = nodes >= (1L << 14) && (50 * by_two <= 49 * 8L * nsm || nodes >= 800000);
     const bool f64 = p->precision == LBM_F64, f16 = p->precision == LBM_F32_STORE_F16;
     // (a grid has at most 65535 rows of blocks)
     const bool narrow = p->block_x <= 0 && p->block_y <= 0 && p->ny < 60000 && !f16 && (f64 || nodes < (1L << 20));
     h->bx = p->block_x > 0 ? p->block_x : (p->nx <= 128 || narrow ? 32 : 64);
-    h->by = p->block_y > 0 ? p->block_y : narrow ? (f64 || nodes < 100000 ? 1 : 2) : (h->bx >= 128 ? 1 : 128 / h->bx);
-    h->npt = p->nodes_per_thread > 0 ? p->nodes_per_thread : f64 ? (nodes < (1L << 14) ? 1 : 2) : 3;
+    const int rows = f64 ? (two || nodes < 110000 ? 1 : 4) : nodes < 100000 ? 1 : 2;
+    h->by = p->block_y > 0 ? p->block_y : narrow ? rows : (h->bx >= 128 ? 1 : 128 / h->bx);
+    h->npt = p->nodes_per_thread > 0 ? p->nodes_per_thread : f64 ? (two ? 2 : 1) : 3;
     if (h->bx * h->by > 256 || h->bx <= 0 || h->by <= 0 || h->npt > 3) {
         delete h;
         return fail(nullptr, LBM_ERR_ARG, "block_x * block_y must be <= 256 and nodes_per_thread 1, 2 or 3");

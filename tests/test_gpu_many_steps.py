@@ -110,3 +110,21 @@ def test_divergence_between_two_steps_of_a_launch_is_flagged(size):
     c.step(9)
     assert c.query()[1] == _lib.LBM_ERR_DIVERGED
     c.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(127, 128), (257, 257), (260, 263), (333, 331), (903, 897)])
+def test_fp64_default_shapes_leave_the_same_bits(nx, ny):
+    """FP64 takes one or two nodes per thread by the size of the lattice; both on
+    either side of each line give what one node per thread gives."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1308_2071_gb300 import Cavity
+
+    got = []
+    for shape in ({}, dict(block_x=64, block_y=1, nodes_per_thread=1)):
+        with Cavity(nx, ny, Ra=1e5, Da=1e-2, phi=0.6, precision="f64", **shape) as c:
+            c.step(12)
+            got.append([a.cpu() for a in c.read_state()] + [c.nusselt()])
+    assert all(torch.equal(a, b) for a, b in zip(got[0][:-1], got[1][:-1])) and got[0][-1] == got[1][-1]
