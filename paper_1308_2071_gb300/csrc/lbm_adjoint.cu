@@ -167,7 +167,7 @@ struct Divider {
 // pair, 202 of them arithmetic; 1.35 waves of 20 warps per SM).  512^2 FP32, us
 // per reverse step alone: 7.6; 8.3 with an index per access, and 23.4 for the
 // direct formulas in one kernel for the interior and one for the ring of nodes
-// near the walls on a stream of its own.  The gradient of 600 steps: 19.8 -> 10.2 ms.
+// near the walls on a stream of its own.  The gradient of 600 steps: 19.8 -> 9.8 ms.
 template <class T>
 __global__ void __launch_bounds__(kAdjThreads, sizeof(typename T::R) == 4 ? kAdjBlocks : 2)
     k_adjoint(Src<T> state, const typename T::R* Mnext, typename T::R* Mcur, const typename T::P* __restrict__ phi,

@@ -998,19 +998,16 @@ int lbm_adjoint_step(lbm_handle h, long nsteps, long ckpt_every, double* J, void
     const long K = std::min({ckpt_every, N, best});
     const long nseg = (N + K - 1) / K;
     const size_t rsz = h->precision == LBM_F64 ? sizeof(double) : sizeof(float);
-    void *ckpt = nullptr, *seg = nullptr, *madj = nullptr;
-    double* gphi = nullptr;
-    auto release = [&]() {
-        if (ckpt) cudaFree(ckpt);
-        if (seg) cudaFree(seg);
-        if (madj) cudaFree(madj);
-        if (gphi) cudaFree(gphi);
-    };
-    cudaError_t e = cudaMalloc(&ckpt, (size_t)nseg * h->buf_bytes);
-    // two halves of K - 1 recomputed states: one segment is recomputed while the next is reversed
-    if (e == cudaSuccess && K > 1) e = cudaMalloc(&seg, 2 * (size_t)(K - 1) * h->buf_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&madj, 2 * (size_t)h->gm.plane * NPOP * rsz);
-    if (e == cudaSuccess) e = cudaMalloc(&gphi, sizeof(double) * (size_t)h->p.nx * h->p.ny);
+    // one allocation: kept states, two halves of K - 1 recomputed states (one segment
+    // is recomputed while the next is reversed), two adjoint states, the gradient
+    auto whole = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
+    const size_t of_ckpt = whole((size_t)nseg * h->buf_bytes), of_seg = whole(2 * (size_t)(K - 1) * h->buf_bytes),
+                 of_madj = whole(2 * (size_t)h->gm.plane * NPOP * rsz);
+    char* ckpt = nullptr;
+    auto release = [&]() { cudaFree(ckpt); };
+    cudaError_t e = cudaMalloc(&ckpt, of_ckpt + of_seg + of_madj + sizeof(double) * (size_t)h->p.nx * h->p.ny);
+    void *const seg = ckpt + of_ckpt, *const madj = ckpt + of_ckpt + of_seg;
+    double* const gphi = (double*)(ckpt + of_ckpt + of_seg + of_madj);
     if (e != cudaSuccess) {
         release();
         return cuda_fail(h, e, "adjoint buffers");
@@ -1025,7 +1022,7 @@ int lbm_adjoint_step(lbm_handle h, long nsteps, long ckpt_every, double* J, void
         for (long t = 0; t < N && rc == LBM_OK;) {
             const long j = t + 1;
             const bool copy = j % K == 0 && j <= N - 1;
-            if (copy && (e = cudaMemcpyAsync((char*)ckpt + (size_t)(j / K) * h->buf_bytes, h->buf[h->cur],
+            if (copy && (e = cudaMemcpyAsync(ckpt + (size_t)(j / K) * h->buf_bytes, h->buf[h->cur],
                                              h->buf_bytes, cudaMemcpyDeviceToDevice, h->stream)) != cudaSuccess) {
                 rc = cuda_fail(h, e, "adjoint forward sweep");
                 break;
