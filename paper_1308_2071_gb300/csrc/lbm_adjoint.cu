@@ -45,10 +45,8 @@ __global__ void k_adj_seed(R* __restrict__ M, Geom gm, double L, double dT) {
     }
 }
 
-// Element at a uniform base and a thread's byte offset: one register serves every
-// plane and neighbour, and the planes' bases stay in uniform registers (with an
-// index per access, half of the kernel's instructions were addresses).  The
-// offset fits 32 bits: a lattice of 2^32 bytes per plane takes over 300 GB here.
+// Element at a uniform base and a thread's byte offset (as at() above does for a
+// node's offset).
 template <class S> __device__ __forceinline__ S* at(S* base, unsigned bytes) {
     if constexpr (std::is_const<S>::value) return (S*)((const char*)base + bytes);
     else return (S*)((char*)base + bytes);
@@ -81,13 +79,13 @@ __device__ __forceinline__ void tape_at(const Coef<typename T::R>& c, const Src<
     d[0] = R(0);
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
-        const int o = off - ey9(i) * gm.pitch - ex9(i);
-        d[i] = in_plane(gm, o) ? Conv<typename T::SF, R, T::cg>::ld(src.f + i * gm.plane + o) : R(0);
+        const int e = -ey9(i) * gm.pitch - ex9(i);
+        d[i] = in_plane(gm, off + e) ? Conv<typename T::SF, R, T::cg>::ld(at(src.f, i * gm.plane + e, off)) : R(0);
     }
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-        const int o = off - ey9(j) * gm.pitch - ex9(j);
-        h[j] = in_plane(gm, o) ? Conv<typename T::SG, R, T::cg>::ld(src.g + j * gm.plane + o) : R(0);
+        const int e = -ey9(j) * gm.pitch - ex9(j);
+        h[j] = in_plane(gm, off + e) ? Conv<typename T::SG, R, T::cg>::ld(at(src.g, j * gm.plane + e, off)) : R(0);
     }
     const R F = op::mul(core_frame_in<T>(c.k, src, gm, off, h), c.k.fu);
     tape_node<R, Framed<T>::value>(c.k, (R)phi[off], sums_of(d, h), F, t);

@@ -52,22 +52,27 @@ __device__ __forceinline__ void core_frame_in_x2(const Coll<typename T::R>& k, c
     F0 = F1 = R(0);
     if constexpr (Framed<T>::value) {
         R n0 = R(0), n1 = R(0), s0 = R(0), s1 = R(0);
-        auto pair = [&](int o, R& a, R& b) {
-            if (!in_plane(gm, o, 2)) return;
+        auto pair = [&](int delta, R& a, R& b) {
+            if (!in_plane(gm, off0 + delta, 2)) return;
             if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
-                const char2 v = frame_pair_code<T>(src.t + o);
+                const char2 v = frame_pair_code<T>(at(src.t, delta, off0));
                 a = R((int)(signed char)v.x);
                 b = R((int)(signed char)v.y);
             } else {
-                const auto v = Conv2<typename FrameStore<T>::type, R, T::cg>::ld(src.t + o);
+                const auto v = Conv2<typename FrameStore<T>::type, R, T::cg>::ld(at(src.t, delta, off0));
                 a = v.x;
                 b = v.y;
             }
         };
-        pair(off0, F0, F1);
-        pair(off0 - gm.pitch, s0, s1);  // j = 2: y - 1
-        pair(off0 + gm.pitch, n0, n1);  // j = 4: y + 1
-        const R w = core_frame<T>(src, gm, off0 - 1), e = core_frame<T>(src, gm, off0 + 2);
+        pair(0, F0, F1);
+        pair(-gm.pitch, s0, s1);  // j = 2: y - 1
+        pair(gm.pitch, n0, n1);  // j = 4: y + 1
+        auto one = [&](int delta) {
+            if (!in_plane(gm, off0 + delta)) return R(0);
+            if constexpr (sizeof(typename FrameStore<T>::type) == 1) return R(frame_code<T>(at(src.t, delta, off0)));
+            else return Conv<typename FrameStore<T>::type, R, T::cg>::ld(at(src.t, delta, off0));
+        };
+        const R w = one(-1), e = one(2);
         const R dF = op::sub(F1, F0);
         h0[1] = op::fma(k.w1, op::sub(w, F0), h0[1]);
         h1[1] = op::fma(k.w1, -dF, h1[1]);
@@ -573,7 +578,7 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Coef<float>& c, cons
 #pragma unroll
         for (int j = 1; j < 5; ++j) h[j] = h[j] - c.wt1 * sh;
         if constexpr (VEC) {
-            if (in_plane(gm, off0, 2)) frame_st2<T>(dst.t + off0, k0, k1);
+            if (in_plane(gm, off0, 2)) frame_st2<T>(at(dst.t, 0, off0), k0, k1);
         } else {
             if (in_plane(gm, off0)) dst.t[off0] = k0;
             if (in_plane(gm, off1)) dst.t[off1] = k1;
@@ -583,10 +588,10 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Coef<float>& c, cons
         if (in_plane(gm, off0, 2)) {
 #pragma unroll
             for (int i = 0; i < 9; ++i)
-                Conv2<typename T::SF, float, T::cg>::st(dst.f + i * gm.plane + off0, d[i].v.x, d[i].v.y);
+                Conv2<typename T::SF, float, T::cg>::st(at(dst.f, i * gm.plane, off0), d[i].v.x, d[i].v.y);
 #pragma unroll
             for (int j = 0; j < 5; ++j)
-                Conv2<typename T::SG, float, T::cg>::st(dst.g + j * gm.plane + off0, h[j].v.x, h[j].v.y);
+                Conv2<typename T::SG, float, T::cg>::st(at(dst.g, j * gm.plane, off0), h[j].v.x, h[j].v.y);
         }
     } else {
         if (in_plane(gm, off0)) {
@@ -678,8 +683,8 @@ __device__ __forceinline__ void core_fluid_pair(const Coef<typename T::R>& c, co
     const int off0 = y0 * gm.pitch + x0, off1 = y1 * gm.pitch + x1;
     R phi0 = R(1), phi1 = R(1);
     if constexpr (FIELD) {
-        if (in_plane(gm, off0)) phi0 = Conv<typename T::P, R>::ld(phi + off0);
-        if (in_plane(gm, off1)) phi1 = Conv<typename T::P, R>::ld(phi + off1);
+        if (in_plane(gm, off0)) phi0 = Conv<typename T::P, R>::ld(VEC ? at(phi, 0, off0) : phi + off0);
+        if (in_plane(gm, off1)) phi1 = Conv<typename T::P, R>::ld(VEC ? at(phi, 1, off0) : phi + off1);
     }
     typename FrameStore<T>::type k0, k1;
     R l0, l1, t0, t1;  // T - T0 - F and T - T0 of both nodes
@@ -729,11 +734,11 @@ __device__ __forceinline__ void core_fluid_pair(const Coef<typename T::R>& c, co
     }
     if constexpr (VEC) {
         if (in_plane(gm, off0, 2)) {
-            if constexpr (FR) frame_st2<T>(dst.t + off0, k0, k1);
+            if constexpr (FR) frame_st2<T>(at(dst.t, 0, off0), k0, k1);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) Conv2<typename T::SF, R, T::cg>::st(dst.f + i * gm.plane + off0, d0[i], d1[i]);
+            for (int i = 0; i < 9; ++i) Conv2<typename T::SF, R, T::cg>::st(at(dst.f, i * gm.plane, off0), d0[i], d1[i]);
 #pragma unroll
-            for (int j = 0; j < 5; ++j) Conv2<typename T::SG, R, T::cg>::st(dst.g + j * gm.plane + off0, h0[j], h1[j]);
+            for (int j = 0; j < 5; ++j) Conv2<typename T::SG, R, T::cg>::st(at(dst.g, j * gm.plane, off0), h0[j], h1[j]);
         }
     } else if (in_plane(gm, off0) && in_plane(gm, off1)) {
         if constexpr (FR) {
