@@ -345,12 +345,13 @@ int most_steps(lbm_handle h) { return h->tile.steps ? h->tile.steps : h->duo.thr
 
 // Picks the way (FP32 storage only: FP64 is bound by its arithmetic unit, and
 // the states between of FP16 flow have to be rounded).  Measured, us per step
-// with one step per launch / two / a tile on chip: 64^2 2.2 / 3.5 / 1.0, 200^2 2.3 /
-// 3.6 / 1.7, 384^2 3.4 / 5.1 / 3.3, 450^2 3.6 / 5.1 / 4.1, 601 x 397 4.3 / 5.4 / 5.0,
-// 700^2 6.3 / 7.2 / -, 850^2 9.3 / 9.3 / -, 1024^2 16.6 / 13.9 / -, 4096^2 272 / 170 / -.
+// with one step per launch / a tile on chip: 64^2 2.2 / 1.0, 128^2 1.9 / 1.3, 200^2
+// 2.2 / 1.7, 230^2 2.1 / 1.9, 240^2 2.1 / 2.1, 260^2 2.3 / 2.5, 400^2 3.0 / 3.8, 500 x 100
+// 2.1 / 1.9, 1000 x 60 2.1 / 2.1; one / two: 700^2 6.1 / 7.4, 800^2 7.6 / 8.8, 850^2 9.4 /
+// 9.2, 900^2 12.0 / 10.8, 1024^2 16.5 / 13.7, 4096^2 272 / 170.
 cudaError_t choose_steps(lbm_handle h) {
-    constexpr double kTileWorth = 3.2;  // us per step of tile_shape's model (384^2: 3.0, 450^2: 3.8)
-    constexpr long kTwosWorth = 850000;  // nodes
+    constexpr double kTileWorth = 1.8;  // us per step of tile_shape's model (240^2: 1.6, 250^2: 1.8)
+    constexpr long kTwosWorth = 720000;  // nodes
     if (h->precision != PREC_F32 && h->precision != PREC_F32T) return cudaSuccess;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);

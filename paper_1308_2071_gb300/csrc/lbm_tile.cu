@@ -9,16 +9,16 @@
 // Nothing is exchanged between blocks, so no wait is needed; the surround is
 // computed by the neighbours as well.  Two copies of the region alternate in
 // shared memory, with one barrier per step.  Measured, us per step against one
-// step per launch: 64^2 2.9 -> 0.98, 120^2 2.6 -> 1.2, 200^2 3.0 -> 1.7, 250^2 3.1 ->
-// 2.1, 384^2 4.2 -> 3.1, 450^2 4.8 -> 4.1; beyond that the repeated surround costs
-// more than the launches.  Bound by the latency of a node's chain of operations
-// (0.7 us per step) on small lattices, by instruction issue on the larger.
+// step per launch: 64^2 2.2 -> 0.98, 128^2 1.9 -> 1.3, 200^2 2.2 -> 1.7; from 250^2 on the
+// repeated surround costs more than the launches (300^2 2.3 -> 2.7).  Bound by the
+// latency of a node's chain of operations (0.8 us per step) on small lattices, by
+// the FMA pipe on the repeated nodes on the larger: two nodes per thread in paired
+// instructions halve the instructions and gain 3 % at 200^2 but lose 5 % at 64^2
+// (not kept).
 //
 // The tile and the number of steps come from a cost model (tile_shape): larger
 // tiles repeat less of the surround, smaller ones spread over more SMs, and
 // more steps share one launch but need a wider surround.
-#include <math.h>
-
 #include <algorithm>
 
 #include "lbm_internal.h"
@@ -183,19 +183,16 @@ TileShape tile_shape(int nx, int ny, int nsm) {
     TileShape best;
     for (int tx = 1; tx <= std::min(64, nx / kTileLeast); ++tx)
         for (int ty = 1; ty <= std::min(64, ny / kTileLeast); ++ty) {
-            const int tw = (nx + tx - 1) / tx, th = (ny + ty - 1) / ty;
-            const long tiles = (long)tx * ty;
-            if (tiles > 8L * nsm) break;
-            const double waves = ceil((double)tiles / (2.0 * nsm));
-            const double share = std::min(2.0, ceil((double)tiles / nsm));  // blocks on an SM at a time
+            const int tw = (nx + tx - 1) / tx, th = (ny + ty - 1) / ty, tiles = tx * ty;
+            if (tiles > 2 * nsm) break;  // one wave
+            const double issue = kTileIssue * (tiles > nsm ? 2 : 1);  // blocks on an SM
             double t = kTileLaunch;
             for (int k = 1; k <= kTileMostSteps; ++k) {
                 // the region of the k-th step from the last, of an inner tile
                 const int n = (tw + 2 * (k - 1)) * (th + 2 * (k - 1));
                 if (n > kTileNodes) break;
-                const double passes = ceil(n / (double)kTileThreads);
-                t += waves * std::max(kTileLatency * passes, kTileIssue * share * ceil(n / 32.0));
-                if (k >= 2 && t / k < best.us) {
+                t += std::max(kTileLatency * ((n + kTileThreads - 1) / kTileThreads), issue * ((n + 31) / 32));
+                if (k >= 2 && t < best.us * k) {
                     best.us = t / k;
                     best.tx = tx;
                     best.ty = ty;
