@@ -31,15 +31,40 @@ __device__ __forceinline__ void wait_for_previous_step() { asm volatile("griddep
 // (see border_node).  Measured against rows that hold the walls too, us per
 // step: FP64 257^2 31 -> 26, 512^2 92 -> 75, FP32 601 x 397 4.8 -> 4.3.  FP16 flow storage: no such
 // columns, every block takes what it meets.
+//
+// On a lattice far larger than the cache (cols < 0; FP32) a row of blocks takes
+// the border nodes of its own rows, and the first and last rows of blocks the
+// y walls: a border node shares 32-byte sectors with its row, which otherwise
+// reach memory twice.  One step per launch, us: 2048^2 74.9 -> 72.0, 4096^2 282.7 -> 275.1.
 template <class T, bool FIELD, bool OBS, bool PAIRS>
 __device__ __forceinline__ void step_border(const Src<T>& src, const Dst<T>& dst, const typename T::P* __restrict__ phi,
                                             const Geom& gm, const Coef<typename T::R>& c, int* __restrict__ status,
                                             double* __restrict__ obs, int cols) {
-    const int threads = blockDim.x * blockDim.y;
-    const int b = ((blockIdx.x - cols) * gridDim.y + blockIdx.y) * threads + threadIdx.y * blockDim.x + threadIdx.x;
-    if (b >= border_count<PAIRS>(gm.nx, gm.ny)) return;
+    const int threads = blockDim.x * blockDim.y, t = threadIdx.y * blockDim.x + threadIdx.x;
     int x, y;
-    border_node<PAIRS>(b, gm.nx, gm.ny, x, y);
+    if (PAIRS && cols < 0) {
+        const int nbc = border_columns<PAIRS>(gm.nx), own = nbc * (int)blockDim.y, j = blockIdx.y;
+        if (t < own) {
+            const int r = t / nbc, col = t - r * nbc;
+            y = 1 + j * (int)blockDim.y + r;
+            if (y >= gm.ny - 1) return;
+            x = col < 2 ? col : gm.nx - nbc + col;
+        } else {
+            const int m = threads - own, last = (int)gridDim.y - (gm.nx + m - 1) / m;
+            if (j >= last) {
+                x = (j - last) * m + t - own;
+                y = gm.ny - 1;
+            } else {
+                x = j * m + t - own;
+                y = 0;
+            }
+            if (x >= gm.nx) return;
+        }
+    } else {
+        const int b = ((blockIdx.x - cols) * gridDim.y + blockIdx.y) * threads + t;
+        if (b >= border_count<PAIRS>(gm.nx, gm.ny)) return;
+        border_node<PAIRS>(b, gm.nx, gm.ny, x, y);
+    }
     update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x, y, status, obs);
 }
 
@@ -115,7 +140,7 @@ __global__ void __launch_bounds__(256, step_blocks<T>())
     wait_for_previous_step();
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if constexpr (Core<T>::value) {
-        if ((int)blockIdx.x >= cols) {
+        if ((int)blockIdx.x >= abs(cols)) {
             step_border<T, FIELD, OBS, true>(src, dst, phi, gm, c, status, obs, cols);
             return;
         }
@@ -377,7 +402,13 @@ template <> const Coef<float>& coef_of<PrecF32T>(const CoefSet& cs) { return cs.
 template <class T, bool PAIRS, class K>
 static cudaError_t launch_one_step(K k, int gx, int gy, const StepLaunch& L, const Coef<typename T::R>& c, bool field) {
     const int per_col = gy * L.bx * L.by;  // border nodes that a column of blocks holds
-    const int border = Core<T>::value ? (border_count<PAIRS>(L.gm.nx, L.gm.ny) + per_col - 1) / per_col : 0;
+    int border = Core<T>::value ? (border_count<PAIRS>(L.gm.nx, L.gm.ny) + per_col - 1) / per_col : 0;
+    bool spread = false;  // see step_border
+    if (PAIRS && border && (long)L.gm.nx * L.gm.ny >= (1L << 21)) {
+        const int others = L.bx * L.by - border_columns<PAIRS>(L.gm.nx) * L.by;  // threads left for the y walls
+        spread = others > 0 && 2 * ((L.gm.nx + others - 1) / others) <= gy;
+        if (spread) border = 1;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(gx + border, gy);
     cfg.blockDim = dim3(L.bx, L.by);
@@ -389,7 +420,8 @@ static cudaError_t launch_one_step(K k, int gx, int gy, const StepLaunch& L, con
     cfg.attrs = at;
     cfg.numAttrs = L.pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, src_view<T>(L.src, L.gm.plane), dst_view<T>(L.dst, L.gm.plane),
-                              field ? (const typename T::P*)L.phi : nullptr, L.gm, c, L.status, L.obs, gx);
+                              field ? (const typename T::P*)L.phi : nullptr, L.gm, c, L.status, L.obs,
+                              spread ? -gx : gx);
 }
 
 template <class T, bool FIELD, bool OBS>

@@ -11,10 +11,10 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 SMALL = [(5, 5), (6, 11), (8, 8), (9, 8), (17, 13), (64, 64), (65, 33), (66, 9), (129, 41), (190, 12), (257, 70), (7, 900)]
-# two steps per launch from 850,000 nodes: strips of up to 94 pairs, segments of up to 32 rows, wall tiles of 28 and 22 nodes
+# two steps per launch from 720,000 nodes: strips of up to 94 pairs, segments of up to 32 rows, wall tiles of 28 and 22 nodes
 LARGE = [(1024, 832), (1025, 831), (901, 950), (2001, 437), (2003, 439), (8, 110000), (9, 95001), (110003, 8), (88300, 10),
-         (1501, 1500)]
-MIDDLE = [(500, 451), (601, 397)]  # one step per launch
+         (1501, 1500), (848, 850), (851, 849), (7, 103001)]
+MIDDLE = [(250, 249), (500, 451), (601, 397), (847, 849)]  # one step per launch
 SIZES = SMALL + MIDDLE + LARGE
 
 
@@ -54,6 +54,14 @@ def _same(a, b, n):
 def test_steps_in_twos_leave_the_same_bits(size, precision):
     a, b = _pair(*size, precision=precision)
     _same(a, b, 13)
+
+
+# one step per launch: from 2^21 nodes rows of blocks take their own border nodes, if the y walls fit beside them
+@pytest.mark.parametrize("size", [(2049, 1100), (1100, 2003), (300001, 8), (40, 60001), (2048, 1024)])
+@pytest.mark.parametrize("block", [dict(block_x=32, block_y=1), dict(block_x=64, block_y=2), dict(block_x=8, block_y=2)])
+def test_border_nodes_beside_their_rows(size, block):
+    a, b = _pair(*size, **block)
+    _same(a, b, 4)
 
 
 @pytest.mark.parametrize("size", [(70, 50), (1040, 820)])
