@@ -7,9 +7,11 @@ of the whole lattice).  Prints ONE JSON line (rank 0).
 
   value     coupled MLUPS (nodes x steps / s / 1e6), device-resident state,
             CUDA events on the library's stream around exactly --steps steps.
-  roofline  the step kernel (the only kernel in the timed region) against the
-            measured HBM copy bandwidth: algorithmic bytes = every population
-            read once and written once (FP32: 28 x 4 = 112 B per node-step).
+  roofline  the step kernels (the only ones in the timed region) against the
+            measured HBM copy bandwidth: algorithmic bytes of a launch = every
+            population and frame read once and written once (FP32: 114 B per
+            node), whether it takes one step or, as FP32 does on large
+            lattices, two.
   e2e       same metric through the public API from host memory: the initial
             state is loaded from a host checkpoint (H2D), the Nusselt numbers
             of every step are written to pinned host memory (D2H, one
@@ -70,7 +72,10 @@ def parse():
     return ap.parse_args()
 
 
-def kernel_sources_digest(names=("lbm_device.cuh", "lbm_kernels.cu")):
+STEP_SOURCES = ("lbm_device.cuh", "lbm_core.cuh", "lbm_node.cuh", "lbm_kernels.cu", "lbm_duo.cuh", "lbm_duo.cu")
+
+
+def kernel_sources_digest(names=STEP_SOURCES):
     import hashlib
 
     hsh = hashlib.sha256()
@@ -80,7 +85,26 @@ def kernel_sources_digest(names=("lbm_device.cuh", "lbm_kernels.cu")):
     return hsh.hexdigest()[:16]
 
 
-ADJOINT_SOURCES = ("lbm_device.cuh", "lbm_kernels.cu", "lbm_adjoint.cuh", "lbm_adjoint.cu")
+ADJOINT_SOURCES = ("lbm_device.cuh", "lbm_core.cuh", "lbm_node.cuh", "lbm_kernels.cu", "lbm_adjoint.cuh",
+                   "lbm_adjoint.cu")
+# FP32 lattices of this many nodes and more take two steps per launch (choose_steps of lbm_api.cu)
+TWO_STEP_NODES = 720000
+
+
+def steps_per_launch(precision, nodes):
+    """Of the step kernels on a lattice larger than what fits on chip."""
+    return 2 if precision in ("f32", "f32t") and nodes >= TWO_STEP_NODES else 1
+
+
+def step_launches(precision, nodes, steps):
+    """Launches of one lbm_step(steps): graphs of 64 steps, then the rest, of
+    which the last step is a launch of its own.  (A lower bound on the FP32
+    lattices that take several steps per launch on chip.)"""
+    if steps_per_launch(precision, nodes) == 1:
+        return steps
+    graphs = max(0, (steps - 1) // 64)
+    left = steps - 64 * graphs
+    return 32 * graphs + left // 2 + 1 if left else 32 * graphs
 
 
 def recorded_adjoint_instructions():
@@ -94,7 +118,7 @@ def recorded_adjoint_instructions():
     vals = {}
     for line in text.splitlines():
         if ":" in line and line.split(":", 1)[0] in ("kernel_sources_sha256", "warp_instructions_forward",
-                                                      "warp_instructions_k_adjoint", "warp_instructions_k_adjoint_ring"):
+                                                      "warp_instructions_k_adjoint"):
             k, v = line.split(":", 1)
             vals[k] = v.strip()
     if vals.get("kernel_sources_sha256") != kernel_sources_digest(ADJOINT_SOURCES):
@@ -392,8 +416,8 @@ def long_run_leg(n=1024, steps=50000):
 
 def batched_leg(steps, warmup, ncav=256, seed=2071):
     """Batched sweep: ncav cavities of uneven size (64^2..512^2), log-uniform Ra
-    and Da, uniform porosity (seeded draws), FP32, one persistent
-    graph-captured launch per call, autotuned tile shape."""
+    and Da, uniform porosity (seeded draws), FP32, autotuned tile shape and
+    schedule, graph-captured."""
     import torch
 
     from paper_1308_2071_gb300 import Batch
@@ -423,8 +447,10 @@ def batched_leg(steps, warmup, ncav=256, seed=2071):
                            if th == -2 else "runs of node pairs side by side along x" if th == -1 else
                            "runs of consecutive nodes" if th == 0 else "rectangles"),
                 nodes_per_thread=(2 if th < 0 else 1 if (tw if th == 0 else tw * th) in (32, 256) else 2),
-                mode="one persistent cooperative launch per call, graph-captured",
-                blocks=q["nblocks"], tiles=q["ntiles"], launches=1, diverged=int(st.sum()),
+                mode="autotuned schedule, graph-captured: one persistent cooperative launch per call, or one launch "
+                     "per two steps (which reads and writes the lattices once for both; hbm_gbs counts "
+                     "114 B per node and step either way)",
+                blocks=q["nblocks"], tiles=q["ntiles"], diverged=int(st.sum()),
                 status=int(rc), sizes="U{64..512} square, seed %d" % seed)
 
 
@@ -460,13 +486,14 @@ def adjoint_leg(n=512, nsteps=2000, ckpt=100):
     # is not the bound; the kernels are instruction- and latency-bound.  Bound:
     # the instruction issue rate (4 warp instructions per SM per clock at the
     # maximum SM clock) over the warp instructions one gradient executes: the
-    # forward sweep and the recomputation (2 N - ceil(N / K) step launches) and
-    # N reverse steps (interior and wall-ring kernels), per launch from ncu.
+    # forward sweep and the recomputation (2 N - ceil(N / K) step launches; the
+    # library keeps a state at least every sqrt(N / 2) steps) and N reverse
+    # steps, per launch from ncu.
     ins = recorded_adjoint_instructions()
     if ins:
-        nseg = -(-nsteps // ckpt)
+        nseg = -(-nsteps // min(ckpt, max(1, round((nsteps / 2) ** 0.5))))
         total = ((2 * nsteps - nseg) * ins["warp_instructions_forward"]
-                 + nsteps * (ins["warp_instructions_k_adjoint"] + ins["warp_instructions_k_adjoint_ring"]))
+                 + nsteps * ins["warp_instructions_k_adjoint"])
         nsm = torch.cuda.get_device_properties(0).multi_processor_count
         try:
             mhz = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["sm_max_mhz"])
@@ -518,7 +545,7 @@ def heterogeneous_leg(n=8192, steps=1000, warmup=3):
         ms = e0.elapsed_time(e1)
         obs = cav.observables(fields=True)
         bpn = BYTES_PER_NODE[prec] + (16 if prec == "f64" else 8) // 2  # + the porosity read
-        gbs = n * n * bpn / (ms * 1e-3 / (steps - warmup)) / 1e9
+        gbs = n * n * bpn / (ms * 1e-3 / (steps - warmup) * steps_per_launch(prec, n * n)) / 1e9
         out[prec] = dict(mlups=round(n * n * (steps - warmup) / (ms * 1e-3) / 1e6, 2), hbm_gbs=round(gbs, 1),
                          hbm_frac=round(gbs / peak, 4), nu_hot=obs["nu_hot"])
         fields[prec] = {k: obs[k].double() for k in ("ux", "uy", "T")}
@@ -600,20 +627,21 @@ def main():
     nodes = a.size * a.size
     mlups = replica_mlups(nodes, a.steps, ms, world)
     peak, peak_kind = load_peaks()
-    per_launch_s = ms * 1e-3 / a.steps
+    together = steps_per_launch(a.precision, nodes)
+    per_launch_s = ms * 1e-3 / a.steps * together
     bpn = BYTES_PER_NODE[a.precision] + (field_bytes(a.precision) if a.field else 0)
     achieved = nodes * bpn / per_launch_s / 1e9
     roof = dict(bound="hbm", achieved=round(achieved, 1), peak=peak, unit="GB/s",
                 frac=round(achieved / peak, 4),
-                traffic=recorded_traffic(a.precision, a.size, a.field), kernel="k_step",
-                algorithmic_bytes_per_launch=nodes * bpn, peak_source=peak_kind)
+                traffic=recorded_traffic(a.precision, a.size, a.field), kernel="k_duo" if together == 2 else "k_step",
+                steps_per_launch=together, algorithmic_bytes_per_launch=nodes * bpn, peak_source=peak_kind)
     line = dict(metric=METRIC, value=round(mlups, 2), unit="MLUPS", n_gpus=world, steps=a.steps,
                 warmup=a.warmup, ms_per_step=round(ms / a.steps, 5), higher_is_better=True, scaling="weak",
                 vs_baseline=None, dtype=DTYPE[a.precision], storage=STORAGE[a.precision],
                 data="synthetic (seeded, no dataset)",
                 config=dict(workload(a.size, a.field), parallelism="replicas" if world > 1 else "single GPU",
                             replicas=world),
-                roofline=roof, clocks=clocks, gpu_launches=a.steps, launch_shape=shapes.get(a.precision),
+                roofline=roof, clocks=clocks, gpu_launches=step_launches(a.precision, nodes, a.steps), launch_shape=shapes.get(a.precision),
                 nu_hot_at_end=obs["nu_hot"], status=obs["status"])
     if world > 1 and not a.no_extras and not a.field:
         # every replica runs the end-to-end leg; the job's figure takes the slowest
@@ -630,7 +658,7 @@ def main():
         for prec in ("f64", "f16", "f32t"):
             ms_p, obs_p, _ = device_leg(a.size, prec, k, a.warmup, 1, gpu_index=local,
                                         sample_clocks=False, shapes=shapes)
-            ach = nodes * BYTES_PER_NODE[prec] / (ms_p * 1e-3 / k) / 1e9
+            ach = nodes * BYTES_PER_NODE[prec] / (ms_p * 1e-3 / k * steps_per_launch(prec, nodes)) / 1e9
             variants[prec] = dict(mlups=round(nodes * k / (ms_p * 1e-3) / 1e6, 2),
                                   hbm_gbs=round(ach, 1), hbm_frac=round(ach / peak, 4), steps=k,
                                   nu_hot=obs_p["nu_hot"], nu_cold=obs_p["nu_cold"], at_step=nsteps_cmp,

@@ -85,7 +85,7 @@ typedef struct {
     int thermal_bc;      /* LBM_BC_SIDE_HEATED or LBM_BC_COOLED                          */
     int adiabatic_order; /* 1: T_b = T_f on adiabatic walls; 2: T_b = (4T_f - T_ff)/3   */
     int collision;       /* LBM_MRT or LBM_LBGK                                          */
-    int block_x, block_y;/* launch shape of the step kernel; 0 = library default        */
+    int block_x, block_y;/* launch shape of the one-step kernel; 0 = library default    */
     int nodes_per_thread;/* 1: one node per thread; 2: two along y; 3: two side by side
                             along x (paired loads and stores); 0 = library default */
     double RaI;          /* internal Rayleigh number (Section 2); 0 = none.  With
@@ -153,7 +153,7 @@ int lbm_bounds_check(int* enabled, long* count);
  * divergence flag.  Errors: LBM_ERR_ARG (NULL), LBM_ERR_CUDA. */
 int lbm_reset(lbm_handle h);
 
-/* Autotuner of the step kernel: times candidate launch shapes (block_x x
+/* Autotuner of the one-step kernel: times candidate launch shapes (block_x x
  * block_y threads, nodes_per_thread 1, 2 or 3) on this lattice, keeps the
  * fastest and records it in a text cache at cache_path (NULL: no cache; one
  * line per device, precision, lattice size and porosity mode); a cached entry
@@ -163,7 +163,10 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
 
 /* Advances nsteps time steps of Eq. 17-18 and Eq. 34-35 with the wall rule
  * (Section 4), asynchronously on the handle's stream.  Long runs replay a
- * captured CUDA graph.  Errors: LBM_ERR_ARG (nsteps < 0), LBM_ERR_CUDA. */
+ * captured CUDA graph.  FP32 lattices that fit on chip, and those too large for
+ * the cache, take several steps per launch (the same bits; the last step of a
+ * call is always a launch of its own).  Errors: LBM_ERR_ARG (nsteps < 0),
+ * LBM_ERR_CUDA. */
 int lbm_step(lbm_handle h, long nsteps);
 
 /* Computes the observables of the current state and, for each non-NULL
@@ -297,21 +300,21 @@ int lbm_observables_noalloc(const lbm_params* p, const void* ckpt_dev, size_t by
 
 /* ---- batched sweep ---------------------------------------------------------
  * Many independent cavities (each its own nx, ny, Ra, Da, porosity, ...; one
- * precision, LBM_F32, LBM_F32_FRAMED or LBM_F64, uniform porosity) advanced together: every
+ * precision, LBM_F32, LBM_F32_FRAMED or LBM_F64, uniform porosity) advanced together: an
  * lbm_batch_step() is ONE persistent cooperative kernel launch that runs all
  * requested steps of all cavities (blocks walk a tile list that covers every
  * cavity; a bounded grid-wide barrier, or in the dataflow schedule bounded
- * per-cavity step counters, order the steps), captured into a CUDA graph on
- * first use and replayed.  Per node it runs the same code as lbm_step: with
- * one node per thread each cavity evolves bit for bit as it would alone with
- * one node per thread, with two it agrees to FP rounding. */
+ * per-cavity step counters, order the steps), or, where lbm_batch_tune finds
+ * that faster (FP32 storage), one launch over all cavities per two steps; either
+ * is captured into a CUDA graph on first use and replayed.  Per node it runs
+ * the same code as lbm_step: each cavity evolves bit for bit as it would alone. */
 typedef struct lbm_batch_s* lbm_batch;
 
 /* p: ncav parameter sets (host); same precision in all.  Initial state as in
  * lbm_init.  Errors: LBM_ERR_ARG (with the cavity index in the message),
  * LBM_ERR_CUDA. */
 int lbm_batch_init(const lbm_params* p, int ncav, void* stream, lbm_batch* out);
-/* Advances every cavity by nsteps (asynchronous, one launch). */
+/* Advances every cavity by nsteps (asynchronous, one graph launch). */
 int lbm_batch_step(lbm_batch b, long nsteps);
 /* Mean Nusselt numbers (Eq. 38) of every cavity into host arrays of ncav
  * doubles (either may be NULL); synchronises. */
@@ -328,8 +331,8 @@ int lbm_batch_read_state(lbm_batch b, int cav, double* f_dev, double* g_dev);
  * leaves the kernel; default 2e7.  Also clears a previous timeout. */
 int lbm_batch_set_wait_limit(lbm_batch b, long long polls);
 /* Autotuner: times candidate tile shapes (tile_w x tile_h nodes, or runs of
- * tile_w nodes with tile_h = 0), blocks per SM and the three schedules (see
- * lbm_batch_set_tiles) on this batch, keeps the fastest, and records it in a
+ * tile_w nodes with tile_h = 0), blocks per SM, the three schedules (see
+ * lbm_batch_set_tiles) and two steps per launch on this batch, keeps the fastest, and records it in a
  * text cache (one line per device, precision and batch shape) at cache_path
  * (NULL: no cache); a cached entry is reused without timing.  Tuning advances
  * the lattices, so the batch is reset to t = 0 afterwards.  Outputs may be

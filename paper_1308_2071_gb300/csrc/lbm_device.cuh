@@ -401,7 +401,7 @@ __device__ __forceinline__ Drag<R> drag_at(const Coef<R>& c, const Geom& gm, con
 // for all threads): the plane's address with delta stays in uniform registers
 // and one 32-bit byte offset serves every access of a node.  (A plane has fewer
 // than 2^31 / 14 nodes, so the offset fits.)  For node pairs, where an index per
-// access made up a fifth of the instructions: us per step 3.40 -> 3.19 on 601 x
+// access made up a fifth of the instructions: us per step 4.55 -> 4.27 on 601 x
 // 397 with a porosity field, 4.25 -> 4.16 on 500^2.  Single nodes keep indices,
 // which the on-chip tiles and FP64 run 0.5 % faster with.
 template <class S> __device__ __forceinline__ const S* at(const S* plane, int delta, int off) {
