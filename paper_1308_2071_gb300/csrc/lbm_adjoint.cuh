@@ -36,7 +36,7 @@ __device__ __forceinline__ void tape_node(const Coll<Scalar<V>>& k, V phi, const
     t.p = por_of<V, true>(k, phi);
     t.r = op::mul(op::sub(V(1), phi), t.p.iphi);
     t.s = s;
-    t.m = velocity<V, FR>(k, t.p, s, F);
+    t.m = velocity<V, FR, true>(k, t.p, s, F);
 }
 
 // Seeds that the collision's transpose meets: of E, D, C (products of u and u -

@@ -188,7 +188,8 @@ void fill_coef(const lbm_params* p, const Derived& dv, Coef<R>* c) {
     const double ip = field ? 1.0 : 1.0 / p->phi;
     const double hs[9] = {1 - s[0] / 2, 1 - s[1] / 2, 1 - s[2] / 2, 1 - s[3] / 2, 1 - s[4] / 2,
                           1 - s[5] / 2, 1 - s[6] / 2, 1 - s[7] / 2, 1 - s[8] / 2};
-    const double c_lin = p->phi * dv.nu / dv.K, c_quad = p->phi * dv.Fphi / sqrt(dv.K);
+    double c_lin = p->phi * dv.nu / dv.K, c_quad = p->phi * dv.Fphi / sqrt(dv.K);
+    if (sizeof(R) == 4) c_lin = std::min(c_lin, 4.0 * (double)kMostDrag);  // see Por
     k.hb = (R)(0.5 * dv.gbeta * (field ? 1.0 : p->phi));
     k.gb = (R)dv.gbeta;
     k.cc = (R)(0.25 * (field ? (double)c->a_lin : c_lin));

@@ -123,6 +123,14 @@ __device__ __forceinline__ float inverse_full(float x) {
 }
 __device__ __forceinline__ double inverse_full(double x) { return inverse(x); }
 __device__ __forceinline__ F2 inverse_full(F2 x) { return F2(inverse_full(x.v.x), inverse_full(x.v.y)); }
+// a, or b where a is larger; a NaN stays one
+__device__ __forceinline__ float at_most(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 at_most(F2 a, float b) { return F2(at_most(a.v.x, b), at_most(a.v.y, b)); }
+__device__ __forceinline__ double at_most(double a, double) { return a; }
 // smallest |v|^2 that root() sees: sqrt(x + tiny) differs from sqrt(x) by less than 1e-18
 __device__ __forceinline__ float tiny(float) { return 1e-37f; }
 __device__ __forceinline__ double tiny(double) { return 1e-36; }
@@ -133,6 +141,10 @@ __device__ __forceinline__ F2 tiny(F2) { return F2(1e-37f); }
 
 // What Eq. 22 needs of a node's porosity: with cc = c_lin / 4 and l1 = c_quad /
 // 2, ec = cc + cc^2, and hb = phi g beta / 2; iphi = 1 / phi.
+//
+// The uniform porosity's cc is held at kMostDrag in FP32 (fill_coef), where u is 1e-19
+// of v, so that S + w, 2 cc^2, stays in the reciprocal's range (see velocity).
+constexpr float kMostDrag = 4.6e18f;
 template <class V> struct Por {
     V hb, cc, ec, l1, iphi;
 };
@@ -203,7 +215,12 @@ template <class V> struct Vel {
 // small terms only, so its rounding scales with the drag per step, not with
 // |u| (a fixed fraction of u per step would be integrated by the slow Darcy
 // relaxation).
-template <class V, bool FR> __device__ __forceinline__ Vel<V> velocity(const Coll<Scalar<V>>& k, const Por<V>& p,
+//
+// FIELD, FP32: w is held below 2^126, whose reciprocal is 0 and would leave the cell
+// without any drag (from cc = 6.5e18 on, a porosity of 1e-9 at Da = 1e-6; the
+// roots overflow at 1.8e19 and the step reports the divergence).  Held there, because the
+// same bound on cc cost the one-step kernels 1.3 % (601 x 397 3.95 -> 4.00 us per step).
+template <class V, bool FR, bool FIELD> __device__ __forceinline__ Vel<V> velocity(const Coll<Scalar<V>>& k, const Por<V>& p,
                                                                        const Sums<V>& s, V F) {
     Vel<V> m;
     m.dTl = op::add(s.n0, k.qhalf);
@@ -214,7 +231,8 @@ template <class V, bool FR> __device__ __forceinline__ Vel<V> velocity(const Col
     m.vm = op::root(op::fma(jx, jx, op::fma(vy, vy, op::tiny(V(0)))));
     const V e = op::fma(p.l1, m.vm, p.ec);
     m.S = op::add(op::root(op::add(V(Scalar<V>(0.25)), e)), V(Scalar<V>(0.5)));
-    const V w = op::fma(p.cc, m.S, e);
+    V w = op::fma(p.cc, m.S, e);
+    if constexpr (FIELD) w = op::at_most(w, 4e37f);
     m.ngd = op::mul(w, op::minus_inverse(op::add(m.S, w)));
     m.dux = op::mul(jx, m.ngd);
     m.duy = op::fma(vy, m.ngd, by);
@@ -222,6 +240,17 @@ template <class V, bool FR> __device__ __forceinline__ Vel<V> velocity(const Col
     m.uy = op::add(jy, m.duy);
     return m;
 }
+
+// Eq. 22's quotient 1 / (l0 + sqrt(l0^2 + l1 |v|)).  1 + ngd is the same number, but
+// its rounding is one of 1: where the drag is strong, little of it is right, or
+// nothing (FP32: off by a percent or two at cc = 1e5, 0 or negative from 1e7 on).
+template <class V> __device__ __forceinline__ V quotient(const Por<V>& p, const Vel<V>& m) {
+    return op::inverse(op::add(p.cc, m.S));
+}
+// Whether the drag takes more than half of v (ngd < -1/2; a NaN may count as either), by the bits:
+// off the FP64 unit.
+__device__ __forceinline__ bool strong_drag(float ngd) { return __float_as_uint(ngd) > 0xBF000000u; }
+__device__ __forceinline__ bool strong_drag(double ngd) { return (uint32_t)__double2hiint(ngd) >= 0xBFE00000u; }
 
 // ---- collision -------------------------------------------------------------------------
 
@@ -280,9 +309,10 @@ __device__ __forceinline__ bool too_fast(const Vel<F2>& m) {
     const F2 u = op::fma(m.vm, m.ngd, m.vm);
     return !(u.v.x < 0.5f) || !(u.v.y < 0.5f);
 }
-// FP64: the sign and exponent word decides, off the FP64 unit (|u| is not negative; a NaN is above)
+// FP64: the exponent word decides, off the FP64 unit (a NaN is above).  Without its sign: under
+// strong drag the sum may round to a negative number, of the size of |v| 2^-52.
 __device__ __forceinline__ bool too_fast(const Vel<double>& m) {
-    return (uint32_t)__double2hiint(op::fma(m.vm, m.ngd, m.vm)) >= 0x3FE00000u;
+    return (__double2hiint(op::fma(m.vm, m.ngd, m.vm)) & 0x7FFFFFFF) >= 0x3FE00000;
 }
 
 // Collision of a fluid node, in place on the pulled populations.

@@ -106,7 +106,7 @@ __device__ __forceinline__ void duo_march(const Src<T>& src, const Dst<T>& dst, 
     auto fluid = [&](Pair& p, ST& q0, ST& q1) {
         const Por<F2> por = por_of<F2, FIELD>(k, p.phi);
         const Sums<F2> s = sums_of(p.d, p.h);
-        const Vel<F2> v = velocity<F2, true>(k, por, s, op::mul(k.fu, p.c));
+        const Vel<F2> v = velocity<F2, true, FIELD>(k, por, s, op::mul(k.fu, p.c));
         if (out && too_fast(v)) atomicOr(status, 1);
         F2 next;
         const F2 shift = frame_next<T>(k, v.dT, p.c, next, q0, q1);

@@ -340,7 +340,7 @@ __device__ __forceinline__ Post<typename T::R> core_post(const Coll<typename T::
     const R phi_f = FIELD ? (in_plane(gm, offf) ? Conv<typename T::P, R>::ld(phi + offf) : R(1)) : R(0);
     p.por = por_of<R, FIELD>(k, phi_f);
     p.s = sums_of(d, h);
-    p.v = velocity<R, FR>(k, p.por, p.s, op::mul(Ff, k.fu));
+    p.v = velocity<R, FR, FIELD>(k, p.por, p.s, op::mul(Ff, k.fu));
     p.F = Ff;
     p.dTl = p.v.dTl;
     p.dT = p.v.dT;
@@ -390,10 +390,19 @@ __device__ __forceinline__ Macro<typename T::R> node_state(const Coef<typename T
     if constexpr (Core<T>::value) {
         const Post<R> p = core_post<T, FIELD>(c.k, gm, BufferSource<T>{c, gm, src}, phi_field, x, y, d, h);
         Macro<R> m;
+        // u and |u| as the step forms them, j + (u - j) and |v| (1 + ngd), or, where the drag takes
+        // more than half of v and they cancel, from the quotient
         const R z = R(0), uu = op::fma(p.v.ux, p.v.ux, op::mul(p.v.uy, p.v.uy));
-        m.ux = p.wall ? z : p.v.ux;
-        m.uy = p.wall ? z : p.v.uy;
-        m.umag = p.wall ? z : op::fma(p.v.vm, p.v.ngd, p.v.vm);
+        m.ux = p.v.ux;
+        m.uy = p.v.uy;
+        m.umag = op::fma(p.v.vm, p.v.ngd, p.v.vm);
+        if (strong_drag(p.v.ngd)) {
+            const R q = quotient(p.por, p.v);
+            m.ux = op::mul(op::add(p.s.ex, p.s.dx), q);
+            m.uy = op::mul(op::fma(p.por.hb, p.v.dT, op::add(p.s.ey, p.s.dy)), q);
+            m.umag = op::mul(p.v.vm, q);
+        }
+        if (p.wall) m.ux = m.uy = m.umag = z;
         m.dP = p.wall ? p.dP : op::fma(R(-0.4), op::mul(uu, p.por.iphi), op::mul(R(0.6), op::add(p.s.a, p.s.b)));
         m.dT = p.dT;
         m.dTl = p.dTl;
@@ -467,7 +476,7 @@ __device__ __forceinline__ void update_fluid(const Coef<typename T::R>& c, const
     const R phi_n = FIELD ? (in_plane(gm, off) ? Conv<typename T::P, R>::ld(phi + off) : R(1)) : R(0);
     const Por<R> p = por_of<R, FIELD>(k, phi_n);
     const Sums<R> s = sums_of(d, h);
-    const Vel<R> v = velocity<R, FR>(k, p, s, op::mul(F, k.fu));
+    const Vel<R> v = velocity<R, FR, FIELD>(k, p, s, op::mul(F, k.fu));
     if (too_fast(v)) atomicOr(status, 1);  // also catches NaN
     typename FrameStore<T>::type code;
     R next;
@@ -698,7 +707,7 @@ __device__ __forceinline__ void core_fluid_pair(const Coef<typename T::R>& c, co
         const F2 F(F0, F1);
         const Por<F2> p = por_of<F2, FIELD>(k, F2(phi0, phi1));
         const Sums<F2> s = sums_of(d, h);
-        const Vel<F2> v = velocity<F2, FR>(k, p, s, op::mul(k.fu, F));
+        const Vel<F2> v = velocity<F2, FR, FIELD>(k, p, s, op::mul(k.fu, F));
         if (too_fast(v)) atomicOr(status, 1);
         F2 shift(0.f, 0.f);
         if constexpr (FR) shift = frame_next<T>(k, v.dT, F, next, k0, k1);
@@ -722,7 +731,7 @@ __device__ __forceinline__ void core_fluid_pair(const Coef<typename T::R>& c, co
         auto node = [&](R (&d)[9], R (&h)[5], R F, R phi_n, typename FrameStore<T>::type& code, R& l, R& t) {
             const Por<R> p = por_of<R, FIELD>(k, phi_n);
             const Sums<R> s = sums_of(d, h);
-            const Vel<R> v = velocity<R, FR>(k, p, s, op::mul(F, k.fu));
+            const Vel<R> v = velocity<R, FR, FIELD>(k, p, s, op::mul(F, k.fu));
             if (too_fast(v)) atomicOr(status, 1);
             R next;
             collide_fluid<R, FIELD, FR>(k, p, s, v, frame_next<T>(k, v.dT, F, next, code), d, h);
