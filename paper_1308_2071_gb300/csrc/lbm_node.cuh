@@ -402,7 +402,8 @@ __device__ __forceinline__ Macro<typename T::R> node_state(const Coef<typename T
             m.uy = op::mul(op::fma(p.por.hb, p.v.dT, op::add(p.s.ey, p.s.dy)), q);
             m.umag = op::mul(p.v.vm, q);
         }
-        if (p.wall) m.ux = m.uy = m.umag = z;
+        if (p.wall) m.ux = m.uy = z;
+        if (m.ux == z && m.uy == z) m.umag = z;  // at rest too: |v| has a floor (see tiny)
         m.dP = p.wall ? p.dP : op::fma(R(-0.4), op::mul(uu, p.por.iphi), op::mul(R(0.6), op::add(p.s.a, p.s.b)));
         m.dT = p.dT;
         m.dTl = p.dTl;
