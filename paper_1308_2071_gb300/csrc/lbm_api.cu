@@ -691,7 +691,7 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
         if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&pr, dev) == cudaSuccess) name = pr.name;
         for (auto& ch : name)
             if (ch == ' ') ch = '_';
-        snprintf(sig, sizeof sig, "step:%s:p%d:%dx%d:f%d", name.c_str(), h->precision, h->p.nx, h->p.ny,
+        snprintf(sig, sizeof sig, "step2:%s:p%d:%dx%d:f%d", name.c_str(), h->precision, h->p.nx, h->p.ny,
                  h->p.use_phi_field);
     }
     int best[3] = {h->bx, h->by, h->npt};
@@ -712,13 +712,15 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
         }
     }
     if (!cached) {
-        const int cand[][3] = {{128, 2, 1}, {64, 4, 1}, {256, 1, 1}, {32, 8, 1}, {32, 1, 1}, {32, 2, 1},
+        // the shape that the handle has (the library's own, if none was given) first
+        const int cand[][3] = {{h->bx, h->by, h->npt},
+                               {128, 2, 1}, {64, 4, 1}, {256, 1, 1}, {32, 8, 1}, {32, 1, 1}, {32, 2, 1},
                                {128, 1, 2}, {64, 2, 2}, {128, 2, 2}, {256, 1, 2}, {32, 4, 2}, {32, 1, 2},
                                {32, 2, 2},  {32, 8, 3}, {64, 4, 3}, {128, 2, 3}, {64, 2, 3}, {128, 1, 3},
                                {256, 1, 3}, {32, 1, 3}, {32, 2, 3}};
-        // below 2^17 nodes one node per thread or two along y: only the last step
-        // of a call runs by itself there (lbm_tile.cu), within 0.3 us of the best
-        const bool few = (long)h->p.nx * h->p.ny < (1L << 17);
+        // on lattices stepped on chip (lbm_tile.cu) one node per thread or two along y: the
+        // one-step kernel takes the last step of a call and the observing ones there
+        const bool few = h->tile.steps != 0;
         cudaEvent_t e0, e1;
         CK(h, cudaEventCreate(&e0));
         CK(h, cudaEventCreate(&e1));
