@@ -399,6 +399,7 @@ constexpr long long kDefaultWaitPolls = 20000000;  // ~2-20 s of 100 ns polls
 // dyn: the schedule of the persistent kernel (0 to 2), plus kInTwos when the
 // steps run two per launch and the persistent kernel takes the last ones.
 constexpr int kInTwos = 3;
+constexpr long kTwosSteps = 64;  // of a graph of two-step launches
 struct TuneChoice {
     int tw = 128, th = 2, blocks_per_sm = 0, dyn = 0;
     int schedule() const { return dyn % kInTwos; }
@@ -445,10 +446,14 @@ struct lbm_batch_s {
     bool split = false;  // k_batch<T, NPT, true>: batch-wide coefficients from the constant bank
     int nblocks = 0;
     long long wait_limit = kDefaultWaitPolls;
-    cudaGraphExec_t gexec = nullptr;
-    long gexec_steps = 0;
-    int gexec_par = -1;
-    long long gexec_limit = -1;
+    // graphs kept between calls, by the parity they start from: the persistent launch, of an
+    // even and of an odd number of steps, and kTwosSteps steps two per launch
+    struct Kept {
+        cudaGraphExec_t exec = nullptr;
+        long steps = 0;
+        long long limit = -1;
+    } kept[2][2];
+    cudaGraphExec_t twos[2] = {nullptr, nullptr};
     std::string err;
     std::string signature;
 };
@@ -685,41 +690,76 @@ int reset(lbm_batch b) {
     return LBM_OK;
 }
 
-void drop_graph(lbm_batch b) {
-    if (b->gexec) cudaGraphExecDestroy(b->gexec);
-    b->gexec = nullptr;
-    b->gexec_steps = 0;
-    b->gexec_par = -1;
+void drop_graphs(lbm_batch b) {
+    for (int par = 0; par < 2; ++par) {
+        for (auto& k : b->kept[par]) {
+            if (k.exec) cudaGraphExecDestroy(k.exec);
+            k.exec = nullptr;
+        }
+        if (b->twos[par]) cudaGraphExecDestroy(b->twos[par]);
+        b->twos[par] = nullptr;
+    }
+}
+
+// Captures what enqueue puts on the capture stream into a graph ready to launch.
+template <class Enqueue> int capture(lbm_batch b, cudaGraphExec_t* exec, Enqueue enqueue) {
+    cudaGraph_t g = nullptr;
+    BCK(b, cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
+    int rc = enqueue(b->cap_stream);
+    cudaError_t e2 = cudaStreamEndCapture(b->cap_stream, &g);
+    if (rc != LBM_OK) {
+        if (g) cudaGraphDestroy(g);
+        return rc;
+    }
+    if (e2 != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("end capture: ") + cudaGetErrorString(e2));
+    cudaGraphExec_t made = nullptr;
+    cudaError_t e = cudaGraphInstantiate(&made, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    *exec = made;
+    return LBM_OK;
+}
+
+// n launches of two steps, from parity par; each flips it
+int enqueue_twos(lbm_batch b, long n, int par, cudaStream_t s) {
+    for (long k = 0; k < n; ++k) {
+        int rc = launch_twos(b, par ^ (int)(k & 1), k > 0, s);
+        if (rc != LBM_OK) return rc;
+    }
+    return LBM_OK;
 }
 
 int run_steps(lbm_batch b, long nsteps, cudaStream_t s) {
     if (nsteps <= 0) return LBM_OK;
-    // two per launch, but for the last one or two steps, which leave B_{n-1}
-    for (bool first = true; b->tune.in_twos() && nsteps >= 3; nsteps -= 2, first = false) {
-        int rc = launch_twos(b, b->par, !first, s);
-        if (rc != LBM_OK) return rc;
-        b->par ^= 1;
-    }
-    const int par = b->par;
-    if (!(b->gexec && b->gexec_steps == nsteps && b->gexec_par == par && b->gexec_limit == b->wait_limit)) {
-        drop_graph(b);
-        cudaGraph_t g = nullptr;
-        BCK(b, cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-        int rc = launch(b, nsteps, par, b->cap_stream);
-        cudaError_t e2 = cudaStreamEndCapture(b->cap_stream, &g);
-        if (rc != LBM_OK) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
+    if (b->tune.in_twos()) {
+        // two per launch, but for the last one or two steps, which leave B_{n-1}: graphs
+        // of kTwosSteps steps (an even number of launches keeps the parity), then the rest
+        for (; nsteps > kTwosSteps; nsteps -= kTwosSteps) {
+            cudaGraphExec_t& g = b->twos[b->par];
+            if (!g) {
+                int rc = capture(b, &g, [&](cudaStream_t c) { return enqueue_twos(b, kTwosSteps / 2, b->par, c); });
+                if (rc != LBM_OK) return rc;
+            }
+            BCK(b, cudaGraphLaunch(g, s));
         }
-        if (e2 != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("end capture: ") + cudaGetErrorString(e2));
-        cudaError_t e = cudaGraphInstantiate(&b->gexec, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-        b->gexec_steps = nsteps;
-        b->gexec_par = par;
-        b->gexec_limit = b->wait_limit;
+        const long pairs = (nsteps - 1) / 2;
+        int rc = enqueue_twos(b, pairs, b->par, s);
+        if (rc != LBM_OK) return rc;
+        b->par ^= (int)(pairs & 1);
+        nsteps -= 2 * pairs;
     }
-    BCK(b, cudaGraphLaunch(b->gexec, s));
+    // calls of the same number of steps start this launch from one parity or from both in
+    // turn: with a graph for either none is instantiated twice
+    lbm_batch_s::Kept& k = b->kept[b->par][nsteps & 1];
+    if (!(k.exec && k.steps == nsteps && k.limit == b->wait_limit)) {
+        if (k.exec) cudaGraphExecDestroy(k.exec);
+        k.exec = nullptr;
+        int rc = capture(b, &k.exec, [&](cudaStream_t c) { return launch(b, nsteps, b->par, c); });
+        if (rc != LBM_OK) return rc;
+        k.steps = nsteps;
+        k.limit = b->wait_limit;
+    }
+    BCK(b, cudaGraphLaunch(k.exec, s));
     if (nsteps & 1) b->par ^= 1;
     return LBM_OK;
 }
@@ -946,7 +986,7 @@ int lbm_batch_tune(lbm_batch b, const char* cache_path, int* tile_w, int* tile_h
         auto trial = [&]() -> int {
             int rc = build_tiles(b);
             if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
-            drop_graph(b);
+            drop_graphs(b);
             if (rc == LBM_OK) rc = run_steps(b, 2, b->stream);  // warm
             if (rc != LBM_OK) return rc;
             BCK(b, cudaEventRecord(e0, b->stream));
@@ -986,7 +1026,7 @@ int lbm_batch_tune(lbm_batch b, const char* cache_path, int* tile_w, int* tile_h
     b->tune = best;
     int rc = build_tiles(b);
     if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
-    drop_graph(b);
+    drop_graphs(b);
     if (rc == LBM_OK) rc = reset(b);  // tuning advanced the lattices: start again from t = 0
     if (rc != LBM_OK) return rc;
     if (tile_w) *tile_w = best.tw;
@@ -1012,7 +1052,7 @@ int lbm_batch_set_tiles(lbm_batch b, int tile_w, int tile_h, int blocks_per_sm, 
     b->tune.dyn = dynamic < 0 || dynamic > 2 ? 0 : dynamic;
     int rc = build_tiles(b);
     if (rc == LBM_OK) rc = grid_size(b, &b->nblocks);
-    drop_graph(b);
+    drop_graphs(b);
     if (rc == LBM_OK) rc = reset(b);
     return rc;
 }
@@ -1028,7 +1068,7 @@ int lbm_batch_query(lbm_batch b, long* t, int* ntiles, int* nblocks) {
 int lbm_batch_destroy(lbm_batch b) {
     if (!b) return LBM_OK;
     if (b->stream) cudaStreamSynchronize(b->stream);
-    drop_graph(b);
+    drop_graphs(b);
     if (b->pool) cudaFree(b->pool);
     if (b->descs) cudaFree(b->descs);
     if (b->tiles) cudaFree(b->tiles);
