@@ -353,10 +353,9 @@ __global__ void __launch_bounds__(256) k_read_state(Src<T> prev, const typename 
     for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
         const int y = (int)(k / gm.nx), x = (int)(k - (long)y * gm.nx);
         R d[9], h[5];
-        Drag<R> dr;
-        const Macro<R> mc = node_state<T, FIELD>(c, gm, prev, phi, x, y, dr, d, h);
         // framed storage: h is relative to T0 + F (F = 0 otherwise)
-        const double Tr = Framed<T>::value ? T0 + (double)mc.F : T0;
+        const R F = node_populations<T, FIELD>(c, gm, prev, phi, x, y, d, h);
+        const double Tr = Framed<T>::value ? T0 + (double)F : T0;
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i * n + k] = w9(i) + (double)d[i];
         g[k] = wt0 * Tr + (double)h[0];
