@@ -123,63 +123,95 @@ int derive(const lbm_params* p, Derived* dv, std::string* why) {
     return LBM_OK;
 }
 
-template <class R>
-void fill_coef(const lbm_params* p, const Derived& dv, Coef<R>* c) {
-    double s[9], z[5];
+struct Rates {
+    double s[9], z[5];  // of the flow and thermal moments (Eq. 20, 31)
+};
+Rates rates_of(const lbm_params* p, const Derived& dv) {
+    Rates r;
     if (p->collision == LBM_LBGK) {
-        for (int k = 0; k < 9; ++k) s[k] = 1.0 / dv.tau_nu;
-        for (int k = 0; k < 5; ++k) z[k] = 1.0 / dv.tau_T;
+        for (int k = 0; k < 9; ++k) r.s[k] = 1.0 / dv.tau_nu;
+        for (int k = 0; k < 5; ++k) r.z[k] = 1.0 / dv.tau_T;
     } else {  // Section 4 choices
-        const double sm[9] = {1.0, 1.1, 1.1, 1.0, 1.2, 1.0, 1.2, 1.0 / dv.tau_nu, 1.0 / dv.tau_nu};
-        const double zm[5] = {1.0, 1.0 / dv.tau_T, 1.0 / dv.tau_T, 1.5, 1.5};
-        memcpy(s, sm, sizeof s);
-        memcpy(z, zm, sizeof z);
+        r = {{1.0, 1.1, 1.1, 1.0, 1.2, 1.0, 1.2, 1.0 / dv.tau_nu, 1.0 / dv.tau_nu},
+             {1.0, 1.0 / dv.tau_T, 1.0 / dv.tau_T, 1.5, 1.5}};
     }
-    for (int k = 0; k < 9; ++k) {
-        c->s[k] = (R)s[k];
-        c->hs[k] = (R)(1.0 - 0.5 * s[k]);
-    }
-    for (int k = 0; k < 5; ++k) {
-        c->z[k] = (R)z[k];
-        c->hz[k] = (R)(1.0 - 0.5 * z[k]);
-    }
-    c->gbeta = (R)dv.gbeta;
-    c->T0 = (R)dv.T0;
-    c->dTh = (R)(p->Th - dv.T0);
-    c->dTc = (R)(p->Tc - dv.T0);
-    c->inv_sigma = (R)(1.0 / p->sigma);
-    c->varpi = (R)p->varpi;
-    c->inv_csT2 = (R)(10.0 / (4.0 + p->varpi));
-    c->wt0 = (R)((1.0 - p->varpi) / 5.0);
-    c->wt1 = (R)((4.0 + p->varpi) / 20.0);
-    c->psi0 = (R)(dv.Q / p->sigma);
-    c->psi3 = (R)(p->varpi * dv.Q / p->sigma);
-    c->qhalf = (R)(0.5 * dv.Q / p->sigma);
-    c->phi = (R)p->phi;
-    c->c_lin = (R)(p->phi * dv.nu / dv.K);  // 0 when Da = INFINITY
-    c->c_quad = (R)(p->phi * dv.Fphi / sqrt(dv.K));
-    // per-cell Ergun (Eq. 5) with d_p^2 fixed by K(phi_bar) = K_bar:
-    // phi nu / K(phi) = 150 nu (1-phi)^2 / (phi^2 d_p^2), phi F_phi / sqrt K = 1.75 (1-phi) / (phi^2 d_p)
+    return r;
+}
+
+// Per-cell Ergun (Eq. 5) with d_p^2 fixed by K(phi_bar) = K_bar:
+// phi nu / K(phi) = 150 nu (1-phi)^2 / (phi^2 d_p^2), phi F_phi / sqrt K = 1.75 (1-phi) / (phi^2 d_p)
+struct Ergun {
+    double lin = 0.0, quad = 0.0;
+};
+Ergun ergun_of(const lbm_params* p, const Derived& dv) {
+    Ergun a;
     if (p->phi < 1.0) {
         const double pb = p->phi;
         const double dp2 = 150.0 * dv.K * (1.0 - pb) * (1.0 - pb) / (pb * pb * pb);
-        c->a_lin = (R)(150.0 * dv.nu / dp2);
-        c->a_quad = (R)(p->forchheimer ? 1.75 / sqrt(dp2) : 0.0);
-    } else {
-        c->a_lin = (R)0;
-        c->a_quad = (R)0;
+        a.lin = 150.0 * dv.nu / dp2;
+        a.quad = p->forchheimer ? 1.75 / sqrt(dp2) : 0.0;
     }
-    // 8-bit temperature frames: the power of two fq whose 128 steps span the
-    // largest |T - T0| expected, the wall temperatures plus the conduction
-    // maximum Q L^2 / (8 alpha_e) of a heat source (alpha_e from A9); a
-    // larger |T - T0| only saturates the frame, which costs precision, not
-    // correctness
+    return a;
+}
+
+// 8-bit temperature frames: the power of two fq whose 128 steps span the
+// largest |T - T0| expected, the wall temperatures plus the conduction
+// maximum Q L^2 / (8 alpha_e) of a heat source (alpha_e from A9); a
+// larger |T - T0| only saturates the frame, which costs precision, not
+// correctness
+double frame_quantum(const lbm_params* p, const Derived& dv) {
     const double alpha = p->sigma * (4.0 + p->varpi) / 10.0 * (dv.tau_T - 0.5);
     const double tspan = fmax(fabs(p->Th - dv.T0), fabs(p->Tc - dv.T0)) + fabs(dv.Q) * dv.L * dv.L / (8.0 * alpha);
-    const double fq = exp2(ceil(log2(tspan / 128.0)));
-    c->fq = (R)fq;
-    c->ifq = (R)(1.0 / fq);
-    c->wt1fq = (R)((4.0 + p->varpi) / 20.0) * (R)fq;
+    return exp2(ceil(log2(tspan / 128.0)));
+}
+
+// The direct form's coefficients (FP16 flow storage).
+void fill_direct(const lbm_params* p, const Derived& dv, Direct* c) {
+    const Rates r = rates_of(p, dv);
+    for (int k = 0; k < 9; ++k) {
+        c->s[k] = (float)r.s[k];
+        c->hs[k] = (float)(1.0 - 0.5 * r.s[k]);
+    }
+    for (int k = 0; k < 5; ++k) {
+        c->z[k] = (float)r.z[k];
+        c->hz[k] = (float)(1.0 - 0.5 * r.z[k]);
+    }
+    c->gbeta = (float)dv.gbeta;
+    c->T0 = (float)dv.T0;
+    c->dTh = (float)(p->Th - dv.T0);
+    c->dTc = (float)(p->Tc - dv.T0);
+    c->inv_sigma = (float)(1.0 / p->sigma);
+    c->varpi = (float)p->varpi;
+    c->inv_csT2 = (float)(10.0 / (4.0 + p->varpi));
+    c->wt0 = (float)((1.0 - p->varpi) / 5.0);
+    c->wt1 = (float)((4.0 + p->varpi) / 20.0);
+    c->psi0 = (float)(dv.Q / p->sigma);
+    c->psi3 = (float)(p->varpi * dv.Q / p->sigma);
+    c->qhalf = (float)(0.5 * dv.Q / p->sigma);
+    c->phi = (float)p->phi;
+    c->c_lin = (float)(p->phi * dv.nu / dv.K);  // 0 when Da = INFINITY
+    c->c_quad = (float)(p->phi * dv.Fphi / sqrt(dv.K));
+    const Ergun a = ergun_of(p, dv);
+    c->a_lin = (float)a.lin;
+    c->a_quad = (float)a.quad;
+    const double fq = frame_quantum(p, dv);
+    c->fq = (float)fq;
+    c->ifq = (float)(1.0 / fq);
+    c->wt1fq = (float)((4.0 + p->varpi) / 20.0) * (float)fq;
+}
+
+template <class R>
+void fill_coef(const lbm_params* p, const Derived& dv, Coef<R>* c) {
+    const Rates r = rates_of(p, dv);
+    const double(&s)[9] = r.s, (&z)[5] = r.z;
+    c->T0 = (R)dv.T0;
+    c->dTh = (R)(p->Th - dv.T0);
+    c->dTc = (R)(p->Tc - dv.T0);
+    c->varpi = (R)p->varpi;
+    c->qhalf = (R)(0.5 * dv.Q / p->sigma);
+    c->phi = (R)p->phi;
+    const Ergun a = ergun_of(p, dv);
+    const double fq = frame_quantum(p, dv);
 
     // the constants of lbm_core.cuh (see there for the rearranged formulas),
     // formed in FP64; with a porosity field 1 / phi comes with the products
@@ -192,9 +224,9 @@ void fill_coef(const lbm_params* p, const Derived& dv, Coef<R>* c) {
     if (sizeof(R) == 4) c_lin = std::min(c_lin, 4.0 * (double)kMostDrag);  // see Por
     k.hb = (R)(0.5 * dv.gbeta * (field ? 1.0 : p->phi));
     k.gb = (R)dv.gbeta;
-    k.cc = (R)(0.25 * (field ? (double)c->a_lin : c_lin));
+    k.cc = (R)(0.25 * (field ? (double)(R)a.lin : c_lin));
     k.ec = field ? (R)0 : (R)(0.25 * c_lin + 0.0625 * c_lin * c_lin);
-    k.l1 = (R)(0.5 * (field ? (double)c->a_quad : c_quad));
+    k.l1 = (R)(0.5 * (field ? (double)(R)a.quad : c_quad));
     k.iphi = (R)(1.0 / p->phi);
     k.niphi = (R)(-1.0 / p->phi);
     k.qhalf = c->qhalf;
@@ -221,7 +253,7 @@ void fill_coef(const lbm_params* p, const Derived& dv, Coef<R>* c) {
     k.s6 = (R)(s[6] / 6);
     k.f5 = (R)(hs[5] / 6);
     k.f6 = (R)(hs[6] / 6);
-    k.is = c->inv_sigma;
+    k.is = (R)(1.0 / p->sigma);
     k.Tis = (R)(dv.T0 / p->sigma);
     k.nis = -k.is;
     k.nTis = -k.Tis;
@@ -291,6 +323,7 @@ int setup_lattice(const lbm_params* p, Derived* dv, CoefSet* cs, Geom* gm, std::
 #endif
     fill_coef<double>(p, *dv, &cs->d);
     fill_coef<float>(p, *dv, &cs->f);
+    fill_direct(p, *dv, &cs->h);
     return LBM_OK;
 }
 }  // namespace lbm

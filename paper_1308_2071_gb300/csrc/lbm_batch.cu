@@ -65,20 +65,7 @@ __device__ __forceinline__ void tile_node(const Tile& tl, int lg_tw, int j, int 
 template <class R>
 __host__ __device__ __forceinline__ Coef<R> with_cavity_rates(const Coef<R>& cu, const Coef<R>& v) {
     Coef<R> c = cu;
-    c.s[7] = v.s[7];
-    c.s[8] = v.s[8];
-    c.hs[7] = v.hs[7];
-    c.hs[8] = v.hs[8];
-    c.z[1] = v.z[1];
-    c.z[2] = v.z[2];
-    c.hz[1] = v.hz[1];
-    c.hz[2] = v.hz[2];
-    c.gbeta = v.gbeta;
     c.phi = v.phi;
-    c.c_lin = v.c_lin;
-    c.c_quad = v.c_quad;
-    c.a_lin = v.a_lin;
-    c.a_quad = v.a_quad;
     c.k.hb = v.k.hb;
     c.k.gb = v.k.gb;
     c.k.cc = v.k.cc;

@@ -308,30 +308,45 @@ template <class R> struct Coll {
     R dTh, dTc, gb;              // wall temperatures minus T0, g beta
 };
 
-// Everything a step needs besides the buffers, in the arithmetic type R.
+// Everything a step needs besides the buffers.  Each storage variant's kernels take
+// what they use: a launch's time grows with its parameters (FP16, 64^2: 0.2 us per
+// step more with both forms' constants in one struct of 408 bytes).
+//
+// FP32 and FP64 storage, in the arithmetic type R.
 template <class R> struct Coef {
     Coll<R> k;
-    R s[9];       // flow relaxation rates (Eq. 20)
-    R hs[9];      // 1 - s_k / 2
-    R z[5];       // thermal relaxation rates (Eq. 31)
-    R hz[5];      // 1 - zeta_k / 2
-    R gbeta;      // g beta (buoyancy G = g beta (T - T0) j, Section 2)
-    R dTh, dTc;   // wall temperatures minus T0
+    R dTh, dTc;  // wall temperatures minus T0
     R T0;
-    R inv_sigma;  // 1 / sigma
-    R varpi;      // D2Q5 constant (Eq. 29)
-    R inv_csT2;   // 1 / c_sT^2 = 10 / (4 + varpi)
-    R wt0, wt1;   // D2Q5 weights w~_0 = (1 - varpi)/5, w~_i = (4 + varpi)/20
-    R psi0, psi3; // Psi_0 = Q/sigma, Psi_3 = varpi Q/sigma (Eq. 30)
-    R qhalf;      // Q / (2 sigma), the source part of Eq. 36
-    R phi;        // uniform porosity
-    R c_lin;      // phi nu / K         (uniform porosity)
-    R c_quad;     // phi F_phi / sqrt K (uniform porosity)
-    R a_lin;      // per-cell: phi nu / K      = a_lin  (1 - phi)^2 / phi^2
-    R a_quad;     // per-cell: phi F_phi / sqrt K = a_quad (1 - phi) / phi^2
-    R fq, ifq;    // 8-bit temperature frames: quantum (a power of two) and its inverse
-    R wt1fq;      // w~_1 fq (exact: fq is a power of two)
+    R varpi;     // D2Q5 constant (Eq. 29)
+    R qhalf;     // Q / (2 sigma), the source part of Eq. 36
+    R phi;       // uniform porosity
 };
+
+// FP16 flow storage: the direct form's.
+struct Direct {
+    float s[9];       // flow relaxation rates (Eq. 20)
+    float hs[9];      // 1 - s_k / 2
+    float z[5];       // thermal relaxation rates (Eq. 31)
+    float hz[5];      // 1 - zeta_k / 2
+    float gbeta;      // g beta (buoyancy G = g beta (T - T0) j, Section 2)
+    float dTh, dTc;   // wall temperatures minus T0
+    float T0;
+    float inv_sigma;  // 1 / sigma
+    float varpi;      // D2Q5 constant (Eq. 29)
+    float inv_csT2;   // 1 / c_sT^2 = 10 / (4 + varpi)
+    float wt0, wt1;   // D2Q5 weights w~_0 = (1 - varpi)/5, w~_i = (4 + varpi)/20
+    float psi0, psi3; // Psi_0 = Q/sigma, Psi_3 = varpi Q/sigma (Eq. 30)
+    float qhalf;      // Q / (2 sigma), the source part of Eq. 36
+    float phi;        // uniform porosity
+    float c_lin;      // phi nu / K         (uniform porosity)
+    float c_quad;     // phi F_phi / sqrt K (uniform porosity)
+    float a_lin;      // per-cell: phi nu / K      = a_lin  (1 - phi)^2 / phi^2
+    float a_quad;     // per-cell: phi F_phi / sqrt K = a_quad (1 - phi) / phi^2
+    float fq, ifq;    // 8-bit temperature frames: quantum (a power of two) and its inverse
+    float wt1fq;      // w~_1 fq (exact: fq is a power of two)
+};
+template <class T> using CoefOf = std::conditional_t<Core<T>::value, Coef<typename T::R>, Direct>;
+static_assert(sizeof(Direct) == 48 * sizeof(float), "what a launch of the direct form carries");
 
 // Geometry of one lattice in one pair of buffers.
 struct Geom {
@@ -367,7 +382,7 @@ template <class R> struct Drag {
 
 // Drag coefficients of one cell from its porosity (FIELD) or the uniform ones.
 template <class R, bool FIELD>
-__device__ __forceinline__ Drag<R> drag_of(const Coef<R>& c, R phi) {
+__device__ __forceinline__ Drag<R> drag_of(const Direct& c, R phi) {
     Drag<R> dr;
     if constexpr (FIELD) {
         R iphi = R(1) / phi;
@@ -387,12 +402,12 @@ __device__ __forceinline__ Drag<R> drag_of(const Coef<R>& c, R phi) {
 }
 
 template <class R, bool FIELD, class P>
-__device__ __forceinline__ Drag<R> drag_at(const Coef<R>& c, const P* phi_field, int off) {
+__device__ __forceinline__ Drag<R> drag_at(const Direct& c, const P* phi_field, int off) {
     if constexpr (FIELD) return drag_of<R, true>(c, Conv<P, R>::ld(phi_field + off));
     return drag_of<R, false>(c, R(0));
 }
 template <class R, bool FIELD, class P>
-__device__ __forceinline__ Drag<R> drag_at(const Coef<R>& c, const Geom& gm, const P* phi_field, int off) {
+__device__ __forceinline__ Drag<R> drag_at(const Direct& c, const Geom& gm, const P* phi_field, int off) {
     if constexpr (FIELD) return drag_at<R, FIELD, P>(c, phi_field, in_plane(gm, off) ? off : 0);
     return drag_of<R, false>(c, R(0));
 }
@@ -414,8 +429,8 @@ template <class S> __device__ __forceinline__ S* at(S* plane, int delta, int off
 // ---- temperature frames -------------------------------------------------------------
 
 // Frame values as stored (FP32) or as 8-bit integers k with F = k fq.
-template <class T, class R>
-__device__ __forceinline__ R frame_ld(const Coef<R>& c, const typename FrameStore<T>::type* p) {
+template <class T, class R = typename T::R>
+__device__ __forceinline__ R frame_ld(const Direct& c, const typename FrameStore<T>::type* p) {
     if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
         const int8_t k = T::cg ? __ldca((const signed char*)p) : __ldg((const signed char*)p);
         return R((int)k) * c.fq;
@@ -427,7 +442,7 @@ __device__ __forceinline__ R frame_ld(const Coef<R>& c, const typename FrameStor
 // The frame a node takes for temperature deviation v, as it will read back,
 // and its stored form.
 template <class T, class R>
-__device__ __forceinline__ R frame_make(const Coef<R>& c, R v, typename FrameStore<T>::type& code) {
+__device__ __forceinline__ R frame_make(const Direct& c, R v, typename FrameStore<T>::type& code) {
     if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
         // a NaN or an overflowing value saturates (the divergence flag reports it)
         const float k = fminf(fmaxf(rintf((float)(v * c.ifq)), -128.f), 127.f);
@@ -451,7 +466,7 @@ __device__ __forceinline__ char2 frame_pair_code(const typename FrameStore<T>::t
 
 // Frames of the node pair (x0, x0 + 1), x0 even.
 template <class T, class R>
-__device__ __forceinline__ void frame_ld2(const Coef<R>& c, const typename FrameStore<T>::type* p, R& a, R& b) {
+__device__ __forceinline__ void frame_ld2(const Direct& c, const typename FrameStore<T>::type* p, R& a, R& b) {
     if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
         const char2 k = T::cg ? __ldca((const char2*)p) : __ldg((const char2*)p);
         a = R((int)(signed char)k.x) * c.fq;
@@ -532,7 +547,7 @@ __device__ __forceinline__ void pull_x2(const Src<T>& src, const Geom& gm, int o
 // and those of the rows above and below come as pairs, the east and west
 // neighbours' as single values.
 template <class T>
-__device__ __forceinline__ void frame_in_x2(const Coef<typename T::R>& c, const Src<T>& src, const Geom& gm,
+__device__ __forceinline__ void frame_in_x2(const Direct& c, const Src<T>& src, const Geom& gm,
                                             int off0, typename T::R (&h0)[5], typename T::R (&h1)[5],
                                             typename T::R& F0, typename T::R& F1) {
     using R = typename T::R;
@@ -580,7 +595,7 @@ __device__ __forceinline__ void frame_in_x2(const Coef<typename T::R>& c, const 
 // (add w~_j (F(x - e_j) - F), j >= 1: nearby frames subtract exactly) and
 // return F.
 template <class T>
-__device__ __forceinline__ typename T::R frame_in(const Coef<typename T::R>& c, const Src<T>& src, const Geom& gm,
+__device__ __forceinline__ typename T::R frame_in(const Direct& c, const Src<T>& src, const Geom& gm,
                                                   int off, typename T::R (&h)[5]) {
     using R = typename T::R;
     if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
@@ -617,10 +632,10 @@ template <class R> struct Macro {
 };
 
 // Eq. 36, Section 2 buoyancy, Eq. 22, Eq. 21, Eq. 23, Eq. 4 at a fluid node.
-// CR: type of the coefficients (R, or float for the node pair F2).  FR: the
+// FR: the
 // thermal values h are relative to the frame F (framed storage).
-template <class R, class CR, bool FR = false>
-__device__ __forceinline__ Macro<R> fluid_macros(const Coef<CR>& c, const Drag<R>& dr,
+template <class R, bool FR = false>
+__device__ __forceinline__ Macro<R> fluid_macros(const Direct& c, const Drag<R>& dr,
                                                  const R (&d)[9], const R (&h)[5], R F = R(0)) {
     Macro<R> m;
     const R n0 = h[0] + h[1] + h[2] + h[3] + h[4];
@@ -666,8 +681,8 @@ __device__ __forceinline__ Macro<R> fluid_macros(const Coef<CR>& c, const Drag<R
 // N^-1 = N^T diag(1/5, 1/2, 1/2, 1/20, 1/4)).  In place on d and h.  FP16 flow
 // storage (and the forward functions the adjoint is checked against); the
 // FP32 and FP64 variants run the increments of lbm_core.cuh.
-template <class R, class CR, bool FR = false>
-__host__ __device__ __forceinline__ void collide(const Coef<CR>& c, R iphi, const Macro<R>& mc, R (&d)[9],
+template <class R, bool FR = false>
+__host__ __device__ __forceinline__ void collide(const Direct& c, R iphi, const Macro<R>& mc, R (&d)[9],
                                         R (&h)[5]) {
     // m = M d (Eq. 9-11), as a deviation from the rest moments
     const R a = (d[1] + d[2]) + (d[3] + d[4]);

@@ -60,10 +60,11 @@ constexpr int kReduceBlocks = 1216;  // 152 SMs x 8; fixed so FP64 sums are repr
 
 enum { PREC_F64 = 0, PREC_F32 = 1, PREC_F16 = 2, PREC_F32T = 3 };
 
-// Coefficients of one lattice in both arithmetic types.
+// Coefficients of one lattice for every storage variant.
 struct CoefSet {
     Coef<double> d;
     Coef<float> f;
+    Direct h;
 };
 
 struct StepLaunch {

@@ -38,7 +38,7 @@ __device__ __forceinline__ void wait_for_previous_step() { asm volatile("griddep
 // reach memory twice.  One step per launch, us: 2048^2 74.9 -> 72.0, 4096^2 282.7 -> 275.1.
 template <class T, bool FIELD, bool OBS, bool PAIRS>
 __device__ __forceinline__ void step_border(const Src<T>& src, const Dst<T>& dst, const typename T::P* __restrict__ phi,
-                                            const Geom& gm, const Coef<typename T::R>& c, int* __restrict__ status,
+                                            const Geom& gm, const CoefOf<T>& c, int* __restrict__ status,
                                             double* __restrict__ obs, int cols) {
     const int threads = blockDim.x * blockDim.y, t = threadIdx.y * blockDim.x + threadIdx.x;
     int x, y;
@@ -70,7 +70,7 @@ __device__ __forceinline__ void step_border(const Src<T>& src, const Dst<T>& dst
 
 template <class T, bool FIELD, bool OBS>
 __global__ void __launch_bounds__(256) k_step(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi,
-                                              Geom gm, Coef<typename T::R> c, int* __restrict__ status,
+                                              Geom gm, CoefOf<T> c, int* __restrict__ status,
                                               double* __restrict__ obs, int cols) {
     wait_for_previous_step();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -106,7 +106,7 @@ template <class T> constexpr int step_blocks() {
 // FP64 would spill under either limit.
 template <class T, bool FIELD, bool OBS>
 __global__ void __launch_bounds__(256, step_blocks<T>())
-    k_step2(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
+    k_step2(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, CoefOf<T> c,
             int* __restrict__ status, double* __restrict__ obs, int cols) {
     wait_for_previous_step();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256, step_blocks<T>())
 // instructions than two nodes apart along y.  Same register cap.
 template <class T, bool FIELD, bool OBS>
 __global__ void __launch_bounds__(256, step_blocks<T>())
-    k_step2x(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
+    k_step2x(Src<T> src, Dst<T> dst, const typename T::P* __restrict__ phi, Geom gm, CoefOf<T> c,
              int* __restrict__ status, double* __restrict__ obs, int cols) {
     wait_for_previous_step();
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256, step_blocks<T>())
 // every warp and an FP64 root per node; 1024^2: 59 us against 87 + 77.
 template <class T, bool FIELD>
 __global__ void __launch_bounds__(256)
-    k_observe(Src<T> prev, const typename T::P* __restrict__ phi, Geom gm, Coef<typename T::R> c,
+    k_observe(Src<T> prev, const typename T::P* __restrict__ phi, Geom gm, CoefOf<T> c,
               typename T::R* ux_out, typename T::R* uy_out, typename T::R* T_out, typename T::R* p_out,
               typename T::R* snap, int snap_valid, double* __restrict__ partials, int nodes, double L, double dT,
               const int* __restrict__ status, unsigned* __restrict__ counter, double* __restrict__ out) {
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256)
 // else they are pulled from B_{n-1} (node_dT); both give the same values.
 template <class T, bool OBS>
 __global__ void __launch_bounds__(32) k_nusselt_rows(Src<T> prev, const double* __restrict__ obs, Geom gm,
-                                                     Coef<typename T::R> c, double L, double dT,
+                                                     CoefOf<T> c, double L, double dT,
                                                      double* __restrict__ partials, unsigned* __restrict__ counter,
                                                      double* __restrict__ out) {
     __shared__ bool last;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(32) k_nusselt_rows(Src<T> prev, const double* 
 // Full FP64 populations of the post-stream state, dense [q][ny][nx].
 template <class T, bool FIELD>
 __global__ void __launch_bounds__(256) k_read_state(Src<T> prev, const typename T::P* __restrict__ phi, Geom gm,
-                                                    Coef<typename T::R> c, double* __restrict__ f,
+                                                    CoefOf<T> c, double* __restrict__ f,
                                                     double* __restrict__ g) {
     using R = typename T::R;
     const long n = (long)gm.nx * gm.ny;
@@ -389,17 +389,17 @@ __global__ void k_convert_phi(const In* __restrict__ in, P* __restrict__ out, Ge
 
 // ---- host launchers ---------------------------------------------------------------
 
-template <class T> static const Coef<typename T::R>& coef_of(const CoefSet& cs);
+template <class T> static const CoefOf<T>& coef_of(const CoefSet& cs);
 template <> const Coef<double>& coef_of<PrecF64>(const CoefSet& cs) { return cs.d; }
 template <> const Coef<float>& coef_of<PrecF32Q>(const CoefSet& cs) { return cs.f; }
-template <> const Coef<float>& coef_of<PrecF16>(const CoefSet& cs) { return cs.f; }
+template <> const Direct& coef_of<PrecF16>(const CoefSet& cs) { return cs.h; }
 template <> const Coef<float>& coef_of<PrecF32T>(const CoefSet& cs) { return cs.f; }
 
 // Launches kernel k with the step's arguments, as a programmatic dependent of
 // the previous work on the stream when L.pdl is set.  gx, gy: blocks over the
 // nodes; PAIRS: which border goes apart.
 template <class T, bool PAIRS, class K>
-static cudaError_t launch_one_step(K k, int gx, int gy, const StepLaunch& L, const Coef<typename T::R>& c, bool field) {
+static cudaError_t launch_one_step(K k, int gx, int gy, const StepLaunch& L, const CoefOf<T>& c, bool field) {
     const int per_col = gy * L.bx * L.by;  // border nodes that a column of blocks holds
     int border = Core<T>::value ? (border_count<PAIRS>(L.gm.nx, L.gm.ny) + per_col - 1) / per_col : 0;
     bool spread = false;  // see step_border
@@ -425,7 +425,7 @@ static cudaError_t launch_one_step(K k, int gx, int gy, const StepLaunch& L, con
 
 template <class T, bool FIELD, bool OBS>
 static cudaError_t launch_step_k(const StepLaunch& L, const CoefSet& cs) {
-    const Coef<typename T::R>& c = coef_of<T>(cs);
+    const CoefOf<T>& c = coef_of<T>(cs);
     const int rows = Core<T>::value ? L.gm.ny - 2 : L.gm.ny;  // the rows without the border, or all
     const int per = L.npt == 2 ? 2 * L.by : L.by, wide = L.npt == 3 ? 2 * L.bx : L.bx;
     const int gx = (L.gm.nx + wide - 1) / wide, gy = (rows + per - 1) / per;

@@ -128,7 +128,7 @@ __device__ __forceinline__ F2 frame_next(const Coll<float>& k, F2 dT, F2 F, F2& 
 
 // Thermal values pulled into node off (framed: in its frame F, in its unit).
 template <class T>
-__device__ __forceinline__ typename T::R pull_heat(const Coef<typename T::R>& c, const Src<T>& src, const Geom& gm,
+__device__ __forceinline__ typename T::R pull_heat(const CoefOf<T>& c, const Src<T>& src, const Geom& gm,
                                                    int off, typename T::R& F) {
     using R = typename T::R;
     R h[5];
@@ -166,7 +166,7 @@ __device__ __forceinline__ Normal normal_of(const Geom& gm, int x, int y) {
 // macroscopic values (u = 0, p_b = p_f, T_b; force phi_b G(T_b) j).  FP16 flow
 // storage; core_wall below is the same rule for FP32 and FP64.
 template <class T, bool FIELD>
-__device__ __forceinline__ Macro<typename T::R> wall_node(const Coef<typename T::R>& c, const Geom& gm,
+__device__ __forceinline__ Macro<typename T::R> wall_node(const Direct& c, const Geom& gm,
                                                           const Src<T>& src, const typename T::P* phi_field,
                                                           int x, int y, Normal nr,
                                                           const Drag<typename T::R>& drb,
@@ -182,7 +182,7 @@ __device__ __forceinline__ Macro<typename T::R> wall_node(const Coef<typename T:
         Fb = in_plane(gm, y * gm.pitch + x) ? frame_ld<T>(c, src.t + y * gm.pitch + x) : R(0);
     }
     const Drag<R> drf = drag_at<R, FIELD, typename T::P>(c, gm, phi_field, offf);
-    const Macro<R> mf = fluid_macros<R, R, FR>(c, drf, df, hf, Ff);
+    const Macro<R> mf = fluid_macros<R, FR>(c, drf, df, hf, Ff);
 
     Macro<R> mb;
     mb.ux = R(0);
@@ -380,14 +380,16 @@ __device__ __forceinline__ void core_collide(const Coll<typename T::R>& k, const
 
 // Post-stream state of node (x, y) (pull + wall rule) and its macroscopic values.
 template <class T, bool FIELD>
-__device__ __forceinline__ Macro<typename T::R> node_state(const Coef<typename T::R>& c, const Geom& gm,
+__device__ __forceinline__ Macro<typename T::R> node_state(const CoefOf<T>& c, const Geom& gm,
                                                            const Src<T>& src, const typename T::P* phi_field,
                                                            int x, int y, Drag<typename T::R>& dr,
                                                            typename T::R (&d)[9], typename T::R (&h)[5]) {
     using R = typename T::R;
     const int off = y * gm.pitch + x;
-    dr = drag_at<R, FIELD, typename T::P>(c, gm, phi_field, off);
     if constexpr (Core<T>::value) {
+        dr.phi = c.phi;
+        if constexpr (FIELD) dr.phi = in_plane(gm, off) ? Conv<typename T::P, R>::ld(phi_field + off) : R(1);
+        dr.iphi = R(1) / dr.phi;
         const Post<R> p = core_post<T, FIELD>(c.k, gm, BufferSource<T>{c, gm, src}, phi_field, x, y, d, h);
         Macro<R> m;
         // u and |u| as the step forms them, j + (u - j) and |v| (1 + ngd), or, where the drag takes
@@ -410,14 +412,15 @@ __device__ __forceinline__ Macro<typename T::R> node_state(const Coef<typename T
         m.F = op::mul(p.F, c.k.fu);
         return m;
     } else {
+    dr = drag_at<R, FIELD, typename T::P>(c, gm, phi_field, off);
     const Normal nr = normal_of(gm, x, y);
     if (nr.dx == 0 && nr.dy == 0) {
         pull<T>(src, gm, off, d, h);
         if constexpr (Framed<T>::value) {
             const R F = frame_in<T>(c, src, gm, off, h);
-            return fluid_macros<R, R, true>(c, dr, d, h, F);
+            return fluid_macros<R, true>(c, dr, d, h, F);
         }
-        return fluid_macros<R, R, false>(c, dr, d, h);
+        return fluid_macros<R, false>(c, dr, d, h);
     }
     return wall_node<T, FIELD>(c, gm, src, phi_field, x, y, nr, dr, d, h);
     }
@@ -427,7 +430,7 @@ __device__ __forceinline__ Macro<typename T::R> node_state(const Coef<typename T
 // ones.  A fluid node needs no macroscopic values for them (FP64 at 1024^2: 75 of 174
 // us of a state read).
 template <class T, bool FIELD>
-__device__ __forceinline__ typename T::R node_populations(const Coef<typename T::R>& c, const Geom& gm,
+__device__ __forceinline__ typename T::R node_populations(const CoefOf<T>& c, const Geom& gm,
                                                           const Src<T>& src, const typename T::P* phi_field, int x,
                                                           int y, typename T::R (&d)[9], typename T::R (&h)[5]) {
     const Normal nr = normal_of(gm, x, y);
@@ -445,7 +448,7 @@ __device__ __forceinline__ typename T::R node_populations(const Coef<typename T:
 // frame mc.F they were computed in, in the node's new frame (T - T0 in the
 // frame's storage type) and stores that frame.
 template <class T>
-__device__ __forceinline__ void frame_out(const Coef<typename T::R>& c, const Geom& gm, const Dst<T>& dst, int off,
+__device__ __forceinline__ void frame_out(const Direct& c, const Geom& gm, const Dst<T>& dst, int off,
                                           const Macro<typename T::R>& mc, typename T::R (&h)[5]) {
     using R = typename T::R;
     typename FrameStore<T>::type code;
@@ -517,7 +520,7 @@ __device__ __forceinline__ void update_fluid(const Coef<typename T::R>& c, const
 // the collision would change where the compiler fuses multiply-adds, and
 // with it the rounding of the lattice.
 template <class T, bool FIELD, bool OBS = false>
-__device__ __forceinline__ void update_node(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& src,
+__device__ __forceinline__ void update_node(const CoefOf<T>& c, const Geom& gm, const Src<T>& src,
                                             const Dst<T>& dst, const typename T::P* phi, int x, int y,
                                             int* status, double* obs = nullptr) {
     using R = typename T::R;
@@ -543,7 +546,7 @@ __device__ __forceinline__ void update_node(const Coef<typename T::R>& c, const 
     Drag<R> dr;
     const Macro<R> mc = node_state<T, FIELD>(c, gm, src, phi, x, y, dr, d, h);
     if (!(mc.umag < R(0.5))) atomicOr(status, 1);  // also catches NaN
-    collide<R, R, Framed<T>::value>(c, dr.iphi, mc, d, h);
+    collide<R, Framed<T>::value>(c, dr.iphi, mc, d, h);
     if constexpr (half_flow<T>()) dither_to_half(d);
     const int off = y * gm.pitch + x;
     if constexpr (Framed<T>::value) frame_out<T>(c, gm, dst, off, mc, h);
@@ -564,7 +567,7 @@ __device__ __forceinline__ void update_node(const Coef<typename T::R>& c, const 
 // VEC: the nodes are x-neighbours off1 = off0 + 1 with x0 even, stored as
 // pairs.
 template <class T, bool OBS = false, bool VEC = false>
-__device__ __forceinline__ void collide_fluid_pair_x2(const Coef<float>& c, const Geom& gm, const Dst<T>& dst,
+__device__ __forceinline__ void collide_fluid_pair_x2(const Direct& c, const Geom& gm, const Dst<T>& dst,
                                                       const float (&a0)[9], const float (&b0)[5],
                                                       const float (&a1)[9], const float (&b1)[5],
                                                       const Drag<float>& r0, const Drag<float>& r1, int off0,
@@ -582,9 +585,9 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Coef<float>& c, cons
     for (int i = 0; i < 9; ++i) d[i] = F2(a0[i], a1[i]);
 #pragma unroll
     for (int j = 0; j < 5; ++j) h[j] = F2(b0[j], b1[j]);
-    const Macro<F2> m = fluid_macros<F2, float, FR>(c, dr, d, h, F2(F0, F1));
+    const Macro<F2> m = fluid_macros<F2, FR>(c, dr, d, h, F2(F0, F1));
     if (!(m.umag.v.x < 0.5f) || !(m.umag.v.y < 0.5f)) atomicOr(status, 1);
-    collide<F2, float, FR>(c, dr.iphi, m, d, h);
+    collide<F2, FR>(c, dr.iphi, m, d, h);
     if constexpr (half_flow<T>()) {
         float v0[9], v1[9];
 #pragma unroll
@@ -648,7 +651,7 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Coef<float>& c, cons
 }
 
 template <class T, bool FIELD, bool OBS = false>
-__device__ __forceinline__ void update_fluid_pair_x2(const Coef<float>& c, const Geom& gm, const Src<T>& src,
+__device__ __forceinline__ void update_fluid_pair_x2(const Direct& c, const Geom& gm, const Src<T>& src,
                                                      const Dst<T>& dst, const typename T::P* phi, int x0, int y0,
                                                      int x1, int y1, int* status, double* obs = nullptr) {
     const int off0 = y0 * gm.pitch + x0, off1 = y1 * gm.pitch + x1;
@@ -794,7 +797,7 @@ __device__ __forceinline__ void core_fluid_pair(const Coef<typename T::R>& c, co
 // any arithmetic (twice the bytes in flight of one node per thread); nodes
 // outside the lattice (valid = false) or on walls take the one-node path.
 template <class T, bool FIELD, bool OBS = false>
-__device__ __forceinline__ void update_pair(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& src,
+__device__ __forceinline__ void update_pair(const CoefOf<T>& c, const Geom& gm, const Src<T>& src,
                                             const Dst<T>& dst, const typename T::P* phi, int x0, int y0,
                                             bool v0, int x1, int y1, bool v1, int* status, double* obs = nullptr) {
     using R = typename T::R;
@@ -840,7 +843,7 @@ __device__ __forceinline__ void update_fluid_xpair(const Coef<typename T::R>& c,
 // as aligned pairs (about a third fewer memory instructions than two nodes
 // apart); otherwise each valid node takes the one-node path.
 template <class T, bool FIELD, bool OBS = false>
-__device__ __forceinline__ void update_xpair(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& src,
+__device__ __forceinline__ void update_xpair(const CoefOf<T>& c, const Geom& gm, const Src<T>& src,
                                              const Dst<T>& dst, const typename T::P* phi, int x0, int y,
                                              int* status, double* obs = nullptr) {
     using R = typename T::R;
@@ -869,7 +872,7 @@ __device__ __forceinline__ void update_xpair(const Coef<typename T::R>& c, const
 // (the wall rule's temperature on wall nodes), in FP64 (framed storage adds
 // the frame to the local part in FP64, so the value keeps its precision).
 template <class T>
-__device__ __forceinline__ double node_dT(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& prev, int x,
+__device__ __forceinline__ double node_dT(const CoefOf<T>& c, const Geom& gm, const Src<T>& prev, int x,
                                           int y) {
     using R = typename T::R;
     const Normal nr = normal_of(gm, x, y);
@@ -908,7 +911,7 @@ __device__ __forceinline__ double node_dT(const Coef<typename T::R>& c, const Ge
 // on the adiabatic rows, taken from the stored rows next to them in the
 // arithmetic node_dT uses, so both give the same bits.
 template <class T>
-__device__ __forceinline__ double obs_dT(const Coef<typename T::R>& c, const Geom& gm, const double* obs, int k,
+__device__ __forceinline__ double obs_dT(const CoefOf<T>& c, const Geom& gm, const double* obs, int k,
                                          int y) {
     using R = typename T::R;
     const int x = k < 5 ? k : gm.nx - 1 - (k - 5);
@@ -979,7 +982,7 @@ __device__ __forceinline__ double slope_cold(const double (&t)[5]) {
 // threads (valid in thread 0): Nu(y) = -L dT/dx / dT, trapezoidal mean over y,
 // FP64.
 template <class T>
-__device__ __forceinline__ void nusselt_block(const Coef<typename T::R>& c, const Geom& gm, const Src<T>& prev,
+__device__ __forceinline__ void nusselt_block(const CoefOf<T>& c, const Geom& gm, const Src<T>& prev,
                                               double L, double dT, double (*sh)[256], double* nu_hot,
                                               double* nu_cold) {
     double w[4] = {0.0, 0.0, 0.0, 0.0};

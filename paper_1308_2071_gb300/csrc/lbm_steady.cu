@@ -19,7 +19,7 @@ namespace lbm {
 // state[0..1]: previous Nu_hot, Nu_cold; [2]: last relative change;
 // [3]: checks done; [4]: stop reason (1 converged, 2 diverged, 3 step cap).
 template <class T>
-__global__ void __launch_bounds__(256) k_steady_check(Src<T> prev, Geom gm, Coef<typename T::R> c, double L,
+__global__ void __launch_bounds__(256) k_steady_check(Src<T> prev, Geom gm, CoefOf<T> c, double L,
                                                        double dT, const int* __restrict__ status, double tol,
                                                        long max_checks, double* __restrict__ state,
                                                        cudaGraphConditionalHandle cond) {
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) k_steady_check(Src<T> prev, Geom gm, Coef
 // psi(x, y) = sum of trapezoids of u_x along y (psi = 0 on the bottom wall).
 template <class T>
 __global__ void __launch_bounds__(256) k_extrema(Src<T> prev, const typename T::P* __restrict__ phi, Geom gm,
-                                                 Coef<typename T::R> c, double* __restrict__ out) {
+                                                 CoefOf<T> c, double* __restrict__ out) {
     using R = typename T::R;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= gm.nx) return;
@@ -69,10 +69,10 @@ __global__ void __launch_bounds__(256) k_extrema(Src<T> prev, const typename T::
     out[3 * x + 2] = pmax;
 }
 
-template <class T> static const Coef<typename T::R>& coef_sel(const CoefSet& cs);
+template <class T> static const CoefOf<T>& coef_sel(const CoefSet& cs);
 template <> const Coef<double>& coef_sel<PrecF64>(const CoefSet& cs) { return cs.d; }
 template <> const Coef<float>& coef_sel<PrecF32Q>(const CoefSet& cs) { return cs.f; }
-template <> const Coef<float>& coef_sel<PrecF16>(const CoefSet& cs) { return cs.f; }
+template <> const Direct& coef_sel<PrecF16>(const CoefSet& cs) { return cs.h; }
 template <> const Coef<float>& coef_sel<PrecF32T>(const CoefSet& cs) { return cs.f; }
 
 template <class T>
