@@ -32,6 +32,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -87,13 +88,12 @@ def kernel_sources_digest(names=STEP_SOURCES):
 
 ADJOINT_SOURCES = ("lbm_device.cuh", "lbm_core.cuh", "lbm_node.cuh", "lbm_kernels.cu", "lbm_adjoint.cuh",
                    "lbm_adjoint.cu")
-# FP32 lattices of this many nodes and more take two steps per launch (choose_steps of lbm_api.cu)
-TWO_STEP_NODES = 720000
 
 
 def steps_per_launch(precision, nodes):
-    """Of the step kernels on a lattice larger than what fits on chip."""
-    return 2 if precision in ("f32", "f32t") and nodes >= TWO_STEP_NODES else 1
+    """Of the step kernels on a square lattice larger than what fits on chip (twos_worth of lbm_api.cu)."""
+    side = math.isqrt(nodes)
+    return 2 if precision in ("f32", "f32t") and side * (side - 9) >= 712000 else 1
 
 
 def step_launches(precision, nodes, steps):

@@ -383,9 +383,20 @@ int most_steps(lbm_handle h) { return h->tile.steps ? h->tile.steps : h->duo.thr
 // 2.2 / 1.7, 230^2 2.1 / 1.9, 240^2 2.1 / 2.1, 260^2 2.3 / 2.5, 400^2 3.0 / 3.8, 500 x 100
 // 2.1 / 1.9, 1000 x 60 2.1 / 2.1; one / two: 700^2 6.1 / 7.4, 800^2 7.6 / 8.8, 850^2 9.4 /
 // 9.2, 900^2 12.0 / 10.8, 1024^2 16.5 / 13.7, 4096^2 272 / 170.
+//
+// Two steps per launch lose on lattices of a few rows, whose wall tiles outweigh the
+// marches (one / two, us per step: 93,750 x 8 9.9 / 16.9, 41,666 x 24 15.4 / 16.3, 62,500 x
+// 24 25.6 / 23.7, 500,000 x 8 71 / 87, 250,000 x 16 68 / 65; the line below is within 10 % of
+// even from 12 rows to 850), and on columns narrower than a march's warps, from 2^21 nodes on, where
+// one step has its border beside its rows, more of them (30 x 33,333 38 / 50, 36 x
+// 27,777 53 / 47, 80 x 50,000 97 / 105, 100 x 40,000 100 / 88).
+bool twos_worth(long nx, long ny) {
+    constexpr long kTwosWorth = 712000, kWallRows = 9;
+    return nx * (ny - kWallRows) >= kTwosWorth && nx >= (nx * ny < (1L << 21) ? 34 : 90);
+}
+
 cudaError_t choose_steps(lbm_handle h) {
     constexpr double kTileWorth = 1.8;  // us per step of tile_shape's model (240^2: 1.6, 250^2: 1.8)
-    constexpr long kTwosWorth = 720000;  // nodes
     if (h->precision != PREC_F32 && h->precision != PREC_F32T) return cudaSuccess;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -397,7 +408,7 @@ cudaError_t choose_steps(lbm_handle h) {
         h->tile = tile;
         return tile_prepare(h->precision, field);
     }
-    if ((long)h->p.nx * h->p.ny >= kTwosWorth) return duo_shape(h->precision, field, h->gm, nsm, &h->duo);
+    if (twos_worth(h->p.nx, h->p.ny)) return duo_shape(h->precision, field, h->gm, nsm, &h->duo);
     return cudaSuccess;
 }
 
