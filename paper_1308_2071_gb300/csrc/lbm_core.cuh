@@ -75,10 +75,11 @@ __device__ __forceinline__ double fms(double a, double b, double c) { return fma
 __device__ __forceinline__ F2 fms(float a, F2 b, F2 c) { return sub(mul(a, b), c); }
 
 // sqrt(x) for x in the normal range (the callers add a floor far below any
-// rounding): the hardware's reciprocal square root y and one Newton step for
-// x - s^2 (FP32, as accurate as sqrtf: 1.0 x 2^-24), or, from its 20-bit FP64
-// form, the series sqrt(x) = t (1 + e/2 + 3 e^2 / 8 + ...) with t = x y and e =
-// 1 - t y of the order of 2^-19 (the next term is below 2^-58).
+// rounding): the hardware's reciprocal square root y, then, in FP32, one step of Newton's
+// method for x - s^2 from s = x y, or, from its 20-bit FP64 form, the binomial series
+// sqrt(x) = t (1 - e)^(-1/2) = t (1 + e/2 + 3 e^2 / 8 + ...) with t = x y and e = 1 - t y of
+// the order of 2^-19.  Relative errors over the callers' arguments at most 1.0 x 2^-24, as a
+// rounded root's, and 1.48 x 2^-53 (inverse: 1.63 x 2^-24 and 1.0 x 2^-53, inverse_full: 1.0).
 __device__ __forceinline__ float root(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -98,9 +99,9 @@ __device__ __forceinline__ F2 root(F2 x) {
     const F2 s = mul(x, F2(y));
     return fma(fma(mul(-1.f, s), s, x), mul(0.5f, F2(y)), s);
 }
-// 1 / x for x near 1: the hardware's approximation (1 ulp in FP32, where the
-// quotient only scales a small correction); in FP64 with the first three
-// terms of 1 / x = y (1 + e + e^2 + ...), e = 1 - x y of the order of 2^-19.
+// 1 / x for normal x, in FP32 below 2^126 (above, the hardware gives 0; see velocity): the
+// hardware's approximation, in FP64 with the first three terms of the geometric series
+// 1 / x = y / (1 - e) = y (1 + e + e^2 + ...), e = 1 - x y of the order of 2^-19.
 __device__ __forceinline__ float inverse(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
