@@ -137,7 +137,6 @@ struct PrecF16 {
     using R = float;
     using P = float;
     static constexpr bool cg = false;
-    static constexpr bool paired = true;  // update_pair computes both nodes with paired FP32 instructions
     static constexpr bool framed = true;
     using ST = int8_t;
 };
@@ -146,12 +145,6 @@ struct PrecF16 {
 // follows the low bits of every value.
 template <class T> struct Core {
     static constexpr bool value = !std::is_same<typename T::SF, __half>::value;
-};
-template <class T, class = void> struct Paired {
-    static constexpr bool value = false;
-};
-template <class T> struct Paired<T, decltype((void)T::paired)> {
-    static constexpr bool value = T::paired;
 };
 template <class T, class = void> struct Framed {
     static constexpr bool value = false;
@@ -249,15 +242,6 @@ __device__ __forceinline__ F2 sqrt(F2 a) { return F2(sqrtf(a.v.x), sqrtf(a.v.y))
 }  // namespace x2
 using x2::F2;
 
-// x and y momentum of deviations d (m_3 and m_5 of Eq. 9-11), with one
-// association of the sums wherever they are taken.
-template <class R> __host__ __device__ __forceinline__ R mom_x(const R (&d)[9]) {
-    return (d[1] - d[3]) + ((d[5] - d[6]) - (d[7] - d[8]));
-}
-template <class R> __host__ __device__ __forceinline__ R mom_y(const R (&d)[9]) {
-    return (d[2] - d[4]) + ((d[5] + d[6]) - (d[7] + d[8]));
-}
-
 // FP16 flow storage: moves each FP32 flow value onto the half-precision grid
 // (13 low mantissa bits cleared) with the rounding threshold taken from the
 // low mantissa bits of two other populations of the node, instead of
@@ -281,7 +265,6 @@ __device__ __forceinline__ void dither_to_half(float (&v)[9]) {
         v[i] = v[i] != v[i] ? v[i] : m;
     }
 }
-template <class T> __host__ __device__ constexpr bool half_flow() { return std::is_same<typename T::SF, __half>::value; }
 
 // ---- per-launch coefficients ----------------------------------------------------
 
@@ -428,30 +411,19 @@ template <class S> __device__ __forceinline__ S* at(S* plane, int delta, int off
 
 // ---- temperature frames -------------------------------------------------------------
 
-// Frame values as stored (FP32) or as 8-bit integers k with F = k fq.
-template <class T, class R = typename T::R>
-__device__ __forceinline__ R frame_ld(const Direct& c, const typename FrameStore<T>::type* p) {
-    if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
-        const int8_t k = T::cg ? __ldca((const signed char*)p) : __ldg((const signed char*)p);
-        return R((int)k) * c.fq;
-    } else {
-        return Conv<typename FrameStore<T>::type, R, T::cg>::ld(p);
-    }
+// FP16 flow storage: a frame is an 8-bit integer k with F = k fq.
+template <class T> __device__ __forceinline__ float frame_ld(const Direct& c, const int8_t* p) {
+    const int8_t k = T::cg ? __ldca((const signed char*)p) : __ldg((const signed char*)p);
+    return (float)(int)k * c.fq;
 }
 
 // The frame a node takes for temperature deviation v, as it will read back,
 // and its stored form.
-template <class T, class R>
-__device__ __forceinline__ R frame_make(const Direct& c, R v, typename FrameStore<T>::type& code) {
-    if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
-        // a NaN or an overflowing value saturates (the divergence flag reports it)
-        const float k = fminf(fmaxf(rintf((float)(v * c.ifq)), -128.f), 127.f);
-        code = (typename FrameStore<T>::type)(int)k;
-        return R(k) * c.fq;
-    } else {
-        code = v;
-        return v;
-    }
+__device__ __forceinline__ float frame_make(const Direct& c, float v, int8_t& code) {
+    // a NaN or an overflowing value saturates (the divergence flag reports it)
+    const float k = fminf(fmaxf(rintf(v * c.ifq), -128.f), 127.f);
+    code = (int8_t)(int)k;
+    return k * c.fq;
 }
 
 // The stored code k of an 8-bit frame (F = k fq), and of a node pair.
@@ -464,19 +436,7 @@ __device__ __forceinline__ char2 frame_pair_code(const typename FrameStore<T>::t
     return T::cg ? __ldca((const char2*)p) : __ldg((const char2*)p);
 }
 
-// Frames of the node pair (x0, x0 + 1), x0 even.
-template <class T, class R>
-__device__ __forceinline__ void frame_ld2(const Direct& c, const typename FrameStore<T>::type* p, R& a, R& b) {
-    if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
-        const char2 k = T::cg ? __ldca((const char2*)p) : __ldg((const char2*)p);
-        a = R((int)(signed char)k.x) * c.fq;
-        b = R((int)(signed char)k.y) * c.fq;
-    } else {
-        const auto v = Conv2<typename FrameStore<T>::type, R, T::cg>::ld(p);
-        a = v.x;
-        b = v.y;
-    }
-}
+// Stores the frames of the node pair (x0, x0 + 1), x0 even.
 template <class T>
 __device__ __forceinline__ void frame_st2(typename FrameStore<T>::type* p, typename FrameStore<T>::type a,
                                           typename FrameStore<T>::type b) {
@@ -547,106 +507,67 @@ __device__ __forceinline__ void pull_x2(const Src<T>& src, const Geom& gm, int o
 // and those of the rows above and below come as pairs, the east and west
 // neighbours' as single values.
 template <class T>
-__device__ __forceinline__ void frame_in_x2(const Direct& c, const Src<T>& src, const Geom& gm,
-                                            int off0, typename T::R (&h0)[5], typename T::R (&h1)[5],
-                                            typename T::R& F0, typename T::R& F1) {
-    using R = typename T::R;
-    if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
-        // 8-bit frames: differences taken on the integers, as in frame_in
-        char2 own = make_char2(0, 0), sth = own, nth = own;
-        signed char w = 0, e = 0;
-        if (in_plane(gm, off0, 2)) own = frame_pair_code<T>(at(src.t, 0, off0));
-        if (in_plane(gm, off0 - gm.pitch, 2)) sth = frame_pair_code<T>(at(src.t, -gm.pitch, off0));  // j = 2: y - 1
-        if (in_plane(gm, off0 + gm.pitch, 2)) nth = frame_pair_code<T>(at(src.t, gm.pitch, off0));  // j = 4: y + 1
-        if (in_plane(gm, off0 - 1)) w = (signed char)frame_code<T>(at(src.t, -1, off0));
-        if (in_plane(gm, off0 + 2)) e = (signed char)frame_code<T>(at(src.t, 2, off0));
-        const int k0 = (signed char)own.x, k1 = (signed char)own.y;
-        h0[1] += c.wt1fq * R((int)w - k0);
-        h1[1] += c.wt1fq * R(k0 - k1);
-        h0[2] += c.wt1fq * R((int)(signed char)sth.x - k0);
-        h1[2] += c.wt1fq * R((int)(signed char)sth.y - k1);
-        h0[3] += c.wt1fq * R(k1 - k0);
-        h1[3] += c.wt1fq * R((int)e - k1);
-        h0[4] += c.wt1fq * R((int)(signed char)nth.x - k0);
-        h1[4] += c.wt1fq * R((int)(signed char)nth.y - k1);
-        F0 = R(k0) * c.fq;
-        F1 = R(k1) * c.fq;
-    } else {
-        R n0 = R(0), n1 = R(0), s0 = R(0), s1 = R(0), w = R(0), e = R(0);
-        F0 = F1 = R(0);
-        if (in_plane(gm, off0, 2)) frame_ld2<T>(c, src.t + off0, F0, F1);
-        if (in_plane(gm, off0 - gm.pitch, 2)) frame_ld2<T>(c, src.t + off0 - gm.pitch, s0, s1);  // j = 2: y - 1
-        if (in_plane(gm, off0 + gm.pitch, 2)) frame_ld2<T>(c, src.t + off0 + gm.pitch, n0, n1);  // j = 4: y + 1
-        if (in_plane(gm, off0 - 1)) w = frame_ld<T>(c, src.t + off0 - 1);
-        if (in_plane(gm, off0 + 2)) e = frame_ld<T>(c, src.t + off0 + 2);
-        h0[1] += c.wt1 * (w - F0);
-        h1[1] += c.wt1 * (F0 - F1);
-        h0[2] += c.wt1 * (s0 - F0);
-        h1[2] += c.wt1 * (s1 - F1);
-        h0[3] += c.wt1 * (F1 - F0);
-        h1[3] += c.wt1 * (e - F1);
-        h0[4] += c.wt1 * (n0 - F0);
-        h1[4] += c.wt1 * (n1 - F1);
-    }
+__device__ __forceinline__ void frame_in_x2(const Direct& c, const Src<T>& src, const Geom& gm, int off0, float (&h0)[5],
+                                            float (&h1)[5], float& F0, float& F1) {
+    using R = float;
+    // differences taken on the integers, as in frame_in
+    char2 own = make_char2(0, 0), sth = own, nth = own;
+    signed char w = 0, e = 0;
+    if (in_plane(gm, off0, 2)) own = frame_pair_code<T>(at(src.t, 0, off0));
+    if (in_plane(gm, off0 - gm.pitch, 2)) sth = frame_pair_code<T>(at(src.t, -gm.pitch, off0));  // j = 2: y - 1
+    if (in_plane(gm, off0 + gm.pitch, 2)) nth = frame_pair_code<T>(at(src.t, gm.pitch, off0));  // j = 4: y + 1
+    if (in_plane(gm, off0 - 1)) w = (signed char)frame_code<T>(at(src.t, -1, off0));
+    if (in_plane(gm, off0 + 2)) e = (signed char)frame_code<T>(at(src.t, 2, off0));
+    const int k0 = (signed char)own.x, k1 = (signed char)own.y;
+    h0[1] += c.wt1fq * R((int)w - k0);
+    h1[1] += c.wt1fq * R(k0 - k1);
+    h0[2] += c.wt1fq * R((int)(signed char)sth.x - k0);
+    h1[2] += c.wt1fq * R((int)(signed char)sth.y - k1);
+    h0[3] += c.wt1fq * R(k1 - k0);
+    h1[3] += c.wt1fq * R((int)e - k1);
+    h0[4] += c.wt1fq * R((int)(signed char)nth.x - k0);
+    h1[4] += c.wt1fq * R((int)(signed char)nth.y - k1);
+    F0 = R(k0) * c.fq;
+    F1 = R(k1) * c.fq;
 }
 
-// Framed storage: thermal values pulled into node off were stored in the
+// FP16 flow storage: thermal values pulled into node off were stored in the
 // frames of the nodes they came from; re-express them in this node's frame F
-// (add w~_j (F(x - e_j) - F), j >= 1: nearby frames subtract exactly) and
-// return F.
+// (add w~_j (F(x - e_j) - F), j >= 1: w~_1 (F_s - F) = (w~_1 fq) (k_s - k), the
+// difference taken on the integers) and return F.
 template <class T>
-__device__ __forceinline__ typename T::R frame_in(const Direct& c, const Src<T>& src, const Geom& gm,
-                                                  int off, typename T::R (&h)[5]) {
-    using R = typename T::R;
-    if constexpr (sizeof(typename FrameStore<T>::type) == 1) {
-        // 8-bit frames: w~_1 (F_s - F) = (w~_1 fq) (k_s - k), the same rounding, the
-        // difference taken on the integers
-        const int k = in_plane(gm, off) ? frame_code<T>(src.t + off) : 0;
+__device__ __forceinline__ float frame_in(const Direct& c, const Src<T>& src, const Geom& gm, int off, float (&h)[5]) {
+    const int k = in_plane(gm, off) ? frame_code<T>(src.t + off) : 0;
 #pragma unroll
-        for (int j = 1; j < 5; ++j) {
-            const int o = off - ey9(j) * gm.pitch - ex9(j);
-            h[j] += c.wt1fq * R((in_plane(gm, o) ? frame_code<T>(src.t + o) : 0) - k);
-        }
-        return R(k) * c.fq;
-    } else {
-        const R F = in_plane(gm, off) ? frame_ld<T>(c, src.t + off) : R(0);
-#pragma unroll
-        for (int j = 1; j < 5; ++j) {
-            const int o = off - ey9(j) * gm.pitch - ex9(j);
-            h[j] += c.wt1 * ((in_plane(gm, o) ? frame_ld<T>(c, src.t + o) : R(0)) - F);
-        }
-        return F;
+    for (int j = 1; j < 5; ++j) {
+        const int o = off - ey9(j) * gm.pitch - ex9(j);
+        h[j] += c.wt1fq * (float)((in_plane(gm, o) ? frame_code<T>(src.t + o) : 0) - k);
     }
+    return (float)k * c.fq;
 }
 
 // ---- macroscopic values -------------------------------------------------------------
 
 template <class R> struct Macro {
     R ux, uy;  // velocity (Eq. 21)
-    R dux, duy;  // u - j, j = (m_3, m_5) of the populations the collision starts from
     R dP;      // phi p - rho0 c_s^2 (Eq. 23)
     R dT;      // T - T0 (Eq. 36)
     R Fx, Fy;  // total force (Eq. 4)
     R umag;    // |u|
-    R F, dTl;  // framed storage: the node's frame and T - T0 - F (else 0 and dT)
+    R F, dTl;  // the node's frame and T - T0 - F (no frames: 0 and dT)
 };
 
-// Eq. 36, Section 2 buoyancy, Eq. 22, Eq. 21, Eq. 23, Eq. 4 at a fluid node.
-// FR: the
-// thermal values h are relative to the frame F (framed storage).
-template <class R, bool FR = false>
-__device__ __forceinline__ Macro<R> fluid_macros(const Direct& c, const Drag<R>& dr,
-                                                 const R (&d)[9], const R (&h)[5], R F = R(0)) {
+// Eq. 36, Section 2 buoyancy, Eq. 22, Eq. 21, Eq. 23, Eq. 4 at a fluid node (R:
+// float, or F2 for a node pair).  The thermal values h are relative to the
+// frame F.
+template <class R>
+__device__ __forceinline__ Macro<R> fluid_macros(const Direct& c, const Drag<R>& dr, const R (&d)[9], const R (&h)[5],
+                                                 R F) {
     Macro<R> m;
     const R n0 = h[0] + h[1] + h[2] + h[3] + h[4];
-    if constexpr (FR) {
-        m.F = F;
-        m.dTl = n0 + c.qhalf;
-        m.dT = F + m.dTl;
-    } else {
-        m.dT = n0 + c.qhalf;
-        m.dTl = m.dT;
-    }
+    m.F = F;
+    m.dTl = n0 + c.qhalf;
+    m.dT = F + m.dTl;
     const R Gy = c.gbeta * m.dT;
     const R jx = (d[1] - d[3]) + (d[5] - d[6]) - (d[7] - d[8]);
     const R jy = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
@@ -661,8 +582,6 @@ __device__ __forceinline__ Macro<R> fluid_macros(const Direct& c, const Drag<R>&
     m.ux = vx * den;
     m.uy = vy * den;
     m.umag = vm * den;
-    m.dux = m.ux - jx;
-    m.duy = m.uy - jy;
     const R uu = m.ux * m.ux + m.uy * m.uy;
     const R s18 = (d[1] + d[2] + d[3] + d[4]) + (d[5] + d[6] + d[7] + d[8]);
     // c_s^2 / (1 - w_0) = 3/5 and rho0 s_0(u) = -(2/3) |u|^2 / phi
@@ -679,11 +598,9 @@ __device__ __forceinline__ Macro<R> fluid_macros(const Direct& c, const Drag<R>&
 // M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4));
 // Eq. 34 with n_eq of Eq. 29 and Psi of Eq. 30, then g+ = N^-1 n+ (Eq. 35,
 // N^-1 = N^T diag(1/5, 1/2, 1/2, 1/20, 1/4)).  In place on d and h.  FP16 flow
-// storage (and the forward functions the adjoint is checked against); the
-// FP32 and FP64 variants run the increments of lbm_core.cuh.
-template <class R, bool FR = false>
-__host__ __device__ __forceinline__ void collide(const Direct& c, R iphi, const Macro<R>& mc, R (&d)[9],
-                                        R (&h)[5]) {
+// storage; the FP32 and FP64 variants run the increments of lbm_core.cuh.
+template <class R>
+__device__ __forceinline__ void collide(const Direct& c, R iphi, const Macro<R>& mc, R (&d)[9], R (&h)[5]) {
     // m = M d (Eq. 9-11), as a deviation from the rest moments
     const R a = (d[1] + d[2]) + (d[3] + d[4]);
     const R b = (d[5] + d[6]) + (d[7] + d[8]);
@@ -748,9 +665,9 @@ __host__ __device__ __forceinline__ void collide(const Direct& c, R iphi, const 
     const R T = c.T0 + mc.dT;
     const R ne1 = ux * T * c.inv_sigma;
     const R ne2 = uy * T * c.inv_sigma;
-    // framed storage: n and the conserved part of n_eq are taken relative to
-    // T0 + F, the flux part (u T / sigma) uses the absolute T
-    const R dTn = FR ? mc.dTl : mc.dT;
+    // n and the conserved part of n_eq are taken relative to T0 + F, the flux
+    // part (u T / sigma) uses the absolute T
+    const R dTn = mc.dTl;
     const R ne3 = c.varpi * dTn;
     const R q0 = (n0 - c.z[0] * (n0 - dTn) + c.hz[0] * c.psi0) * R(0.2);
     const R q1 = (n1 - c.z[1] * (n1 - ne1)) * R(0.5);

@@ -172,17 +172,14 @@ __device__ __forceinline__ Macro<typename T::R> wall_node(const Direct& c, const
                                                           const Drag<typename T::R>& drb,
                                                           typename T::R (&d)[9], typename T::R (&h)[5]) {
     using R = typename T::R;
-    constexpr bool FR = Framed<T>::value;
     const int offf = (y + nr.dy) * gm.pitch + (x + nr.dx);
     R df[9], hf[5];
     pull<T>(src, gm, offf, df, hf);
-    R Ff = R(0), Fb = R(0);  // frames of the inner neighbour and of this wall node
-    if constexpr (FR) {
-        Ff = frame_in<T>(c, src, gm, offf, hf);
-        Fb = in_plane(gm, y * gm.pitch + x) ? frame_ld<T>(c, src.t + y * gm.pitch + x) : R(0);
-    }
+    // frames of the inner neighbour and of this wall node
+    const R Ff = frame_in<T>(c, src, gm, offf, hf);
+    const R Fb = in_plane(gm, y * gm.pitch + x) ? frame_ld<T>(c, src.t + y * gm.pitch + x) : R(0);
     const Drag<R> drf = drag_at<R, FIELD, typename T::P>(c, gm, phi_field, offf);
-    const Macro<R> mf = fluid_macros<R, FR>(c, drf, df, hf, Ff);
+    const Macro<R> mf = fluid_macros<R>(c, drf, df, hf, Ff);
 
     Macro<R> mb;
     mb.ux = R(0);
@@ -195,32 +192,19 @@ __device__ __forceinline__ Macro<typename T::R> wall_node(const Direct& c, const
         mb.dP = mf.dP;
     }
     const bool dirichlet = (gm.thermal_bc == 1) || (nr.dx != 0);
-    if constexpr (FR) {
-        // the wall temperature relative to this node's frame, from differences of nearby frames
-        mb.F = Fb;
-        if (dirichlet) {
-            mb.dTl = ((gm.thermal_bc == 1) ? c.dTc : (x == 0 ? c.dTh : c.dTc)) - Fb;
-        } else if (gm.adi_order == 2) {
-            const int offff = (y + 2 * nr.dy) * gm.pitch + (x + 2 * nr.dx);
-            R Fff;
-            const R dTlff = pull_heat<T>(c, src, gm, offff, Fff) + c.qhalf;
-            mb.dTl = (R(4) * ((Ff - Fb) + mf.dTl) - ((Fff - Fb) + dTlff)) * R(1.0 / 3.0);
-        } else {
-            mb.dTl = (Ff - Fb) + mf.dTl;
-        }
-        mb.dT = Fb + mb.dTl;
+    // the wall temperature relative to this node's frame, from differences of nearby frames
+    mb.F = Fb;
+    if (dirichlet) {
+        mb.dTl = ((gm.thermal_bc == 1) ? c.dTc : (x == 0 ? c.dTh : c.dTc)) - Fb;
+    } else if (gm.adi_order == 2) {
+        const int offff = (y + 2 * nr.dy) * gm.pitch + (x + 2 * nr.dx);
+        R Fff;
+        const R dTlff = pull_heat<T>(c, src, gm, offff, Fff) + c.qhalf;
+        mb.dTl = (R(4) * ((Ff - Fb) + mf.dTl) - ((Fff - Fb) + dTlff)) * R(1.0 / 3.0);
     } else {
-        if (dirichlet) {
-            mb.dT = (gm.thermal_bc == 1) ? c.dTc : (x == 0 ? c.dTh : c.dTc);
-        } else if (gm.adi_order == 2) {
-            const int offff = (y + 2 * nr.dy) * gm.pitch + (x + 2 * nr.dx);
-            R Fff;
-            const R dTff = pull_heat<T>(c, src, gm, offff, Fff) + c.qhalf;
-            mb.dT = (R(4) * mf.dT - dTff) * R(1.0 / 3.0);
-        } else {
-            mb.dT = mf.dT;
-        }
+        mb.dTl = (Ff - Fb) + mf.dTl;
     }
+    mb.dT = Fb + mb.dTl;
     mb.Fx = R(0);
     mb.Fy = drb.phi * c.gbeta * mb.dT;
 
@@ -237,14 +221,10 @@ __device__ __forceinline__ Macro<typename T::R> wall_node(const Direct& c, const
         const R cP = (i == 0) ? R(-5.0 / 3.0) : R(3.0 * w9(i));
         d[i] = df[i] - si + cP * ddP;
     }
-    mb.dux = -mom_x(d);  // u_b = 0
-    mb.duy = -mom_y(d);
-    // g_b = g_eq(T_b, 0) + g_f - g_eq(T_f, u_f) (Eq. 37, first occurrence); framed:
-    // T_b - T_f from the frames' difference and the local parts, the result
-    // re-expressed in this node's frame
+    // g_b = g_eq(T_b, 0) + g_f - g_eq(T_f, u_f) (Eq. 37, first occurrence), in this node's
+    // frame: w~ (T_b - T_f) + w~ (F_f - F_b) = w~ (dTl_b - dTl_f)
     const R Tf = c.T0 + mf.dT;
-    // (framed: w~ (T_b - T_f) + w~ (F_f - F_b) = w~ (dTl_b - dTl_f))
-    const R ddT = FR ? mb.dTl - mf.dTl : mb.dT - mf.dT;
+    const R ddT = mb.dTl - mf.dTl;
     const R adv = Tf * c.inv_sigma * c.inv_csT2 * c.wt1;
     const R sh0 = c.wt0 * ddT;
     const R sh1 = c.wt1 * ddT;
@@ -412,17 +392,14 @@ __device__ __forceinline__ Macro<typename T::R> node_state(const CoefOf<T>& c, c
         m.F = op::mul(p.F, c.k.fu);
         return m;
     } else {
-    dr = drag_at<R, FIELD, typename T::P>(c, gm, phi_field, off);
-    const Normal nr = normal_of(gm, x, y);
-    if (nr.dx == 0 && nr.dy == 0) {
-        pull<T>(src, gm, off, d, h);
-        if constexpr (Framed<T>::value) {
+        dr = drag_at<R, FIELD, typename T::P>(c, gm, phi_field, off);
+        const Normal nr = normal_of(gm, x, y);
+        if (nr.dx == 0 && nr.dy == 0) {
+            pull<T>(src, gm, off, d, h);
             const R F = frame_in<T>(c, src, gm, off, h);
-            return fluid_macros<R, true>(c, dr, d, h, F);
+            return fluid_macros<R>(c, dr, d, h, F);
         }
-        return fluid_macros<R, false>(c, dr, d, h);
-    }
-    return wall_node<T, FIELD>(c, gm, src, phi_field, x, y, nr, dr, d, h);
+        return wall_node<T, FIELD>(c, gm, src, phi_field, x, y, nr, dr, d, h);
     }
 }
 
@@ -444,16 +421,15 @@ __device__ __forceinline__ typename T::R node_populations(const CoefOf<T>& c, co
     return node_state<T, FIELD>(c, gm, src, phi_field, x, y, dr, d, h).F;
 }
 
-// Framed storage: re-expresses the collided thermal values, relative to the
+// FP16 flow storage: re-expresses the collided thermal values, relative to the
 // frame mc.F they were computed in, in the node's new frame (T - T0 in the
 // frame's storage type) and stores that frame.
 template <class T>
 __device__ __forceinline__ void frame_out(const Direct& c, const Geom& gm, const Dst<T>& dst, int off,
-                                          const Macro<typename T::R>& mc, typename T::R (&h)[5]) {
-    using R = typename T::R;
-    typename FrameStore<T>::type code;
-    const R Fn = frame_make<T>(c, mc.dT, code);  // F + dTl as the frame stores it: the new frame
-    const R shift = Fn - mc.F;                    // exact: both are frame values
+                                          const Macro<float>& mc, float (&h)[5]) {
+    int8_t code;
+    const float Fn = frame_make(c, mc.dT, code);  // F + dTl as the frame stores it: the new frame
+    const float shift = Fn - mc.F;                 // exact: both are frame values
     h[0] -= c.wt0 * shift;
 #pragma unroll
     for (int j = 1; j < 5; ++j) h[j] -= c.wt1 * shift;
@@ -473,14 +449,6 @@ constexpr int kObsCols = 10;
 __device__ __forceinline__ void obs_put(const Geom& gm, double* obs, int x, int y, double v) {
     if (x < 5) obs[kObsCols * y + x] = v;
     if (x >= gm.nx - 5) obs[kObsCols * y + 5 + (gm.nx - 1 - x)] = v;
-}
-
-template <class T>
-__device__ __forceinline__ double obs_value(const Macro<typename T::R>& m) {
-    if constexpr (Framed<T>::value)
-        return (double)m.F + (double)m.dTl;
-    else
-        return (double)m.dT;
 }
 
 // One fluid node of the step (FP32 and FP64 storage).
@@ -543,27 +511,26 @@ __device__ __forceinline__ void update_node(const CoefOf<T>& c, const Geom& gm, 
         if constexpr (OBS)
             obs_put(gm, obs, x, y, Framed<T>::value ? (double)op::mul(p.F, c.k.fu) + (double)p.dTl : (double)p.dT);
     } else {
-    Drag<R> dr;
-    const Macro<R> mc = node_state<T, FIELD>(c, gm, src, phi, x, y, dr, d, h);
-    if (!(mc.umag < R(0.5))) atomicOr(status, 1);  // also catches NaN
-    collide<R, Framed<T>::value>(c, dr.iphi, mc, d, h);
-    if constexpr (half_flow<T>()) dither_to_half(d);
-    const int off = y * gm.pitch + x;
-    if constexpr (Framed<T>::value) frame_out<T>(c, gm, dst, off, mc, h);
-    if (in_plane(gm, off)) {
+        Drag<R> dr;
+        const Macro<R> mc = node_state<T, FIELD>(c, gm, src, phi, x, y, dr, d, h);
+        if (!(mc.umag < R(0.5))) atomicOr(status, 1);  // also catches NaN
+        collide<R>(c, dr.iphi, mc, d, h);
+        dither_to_half(d);
+        const int off = y * gm.pitch + x;
+        frame_out<T>(c, gm, dst, off, mc, h);
+        if (in_plane(gm, off)) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) Conv<typename T::SF, R, T::cg>::st(dst.f + i * gm.plane + off, d[i]);
+            for (int i = 0; i < 9; ++i) Conv<typename T::SF, R, T::cg>::st(dst.f + i * gm.plane + off, d[i]);
 #pragma unroll
-        for (int j = 0; j < 5; ++j) Conv<typename T::SG, R, T::cg>::st(dst.g + j * gm.plane + off, h[j]);
-    }
-    if constexpr (OBS) obs_put(gm, obs, x, y, obs_value<T>(mc));
+            for (int j = 0; j < 5; ++j) Conv<typename T::SG, R, T::cg>::st(dst.g + j * gm.plane + off, h[j]);
+        }
+        if constexpr (OBS) obs_put(gm, obs, x, y, (double)mc.F + (double)mc.dTl);
     }
 }
 
-// Two fluid nodes from their pulled values in one pass of F2 arithmetic (FP32
-// arithmetic types only): about half the arithmetic instructions of two nodes.
-// Framed storage: the frames F0, F1 the pulled thermal values b0, b1 are
-// relative to (frame_in), and the frame change of both nodes on the way out.
+// Two fluid nodes from their pulled values in one pass of F2 arithmetic (FP16 flow
+// storage): about half the arithmetic instructions of two nodes.  F0, F1: the
+// frames that the pulled thermal values b0, b1 are relative to (frame_in).
 // VEC: the nodes are x-neighbours off1 = off0 + 1 with x0 even, stored as
 // pairs.
 template <class T, bool OBS = false, bool VEC = false>
@@ -571,10 +538,8 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Direct& c, const Geo
                                                       const float (&a0)[9], const float (&b0)[5],
                                                       const float (&a1)[9], const float (&b1)[5],
                                                       const Drag<float>& r0, const Drag<float>& r1, int off0,
-                                                      int off1, int* status, int x0 = 0, int y0 = 0, int x1 = 0,
-                                                      int y1 = 0, double* obs = nullptr, float F0 = 0.f,
-                                                      float F1 = 0.f) {
-    constexpr bool FR = Framed<T>::value;
+                                                      int off1, int* status, int x0, int y0, int x1, int y1,
+                                                      double* obs, float F0, float F1) {
     Drag<F2> dr;
     dr.phi = F2(r0.phi, r1.phi);
     dr.iphi = F2(r0.iphi, r1.iphi);
@@ -585,10 +550,10 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Direct& c, const Geo
     for (int i = 0; i < 9; ++i) d[i] = F2(a0[i], a1[i]);
 #pragma unroll
     for (int j = 0; j < 5; ++j) h[j] = F2(b0[j], b1[j]);
-    const Macro<F2> m = fluid_macros<F2, FR>(c, dr, d, h, F2(F0, F1));
+    const Macro<F2> m = fluid_macros<F2>(c, dr, d, h, F2(F0, F1));
     if (!(m.umag.v.x < 0.5f) || !(m.umag.v.y < 0.5f)) atomicOr(status, 1);
-    collide<F2, FR>(c, dr.iphi, m, d, h);
-    if constexpr (half_flow<T>()) {
+    collide<F2>(c, dr.iphi, m, d, h);
+    {
         float v0[9], v1[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
@@ -600,20 +565,18 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Direct& c, const Geo
 #pragma unroll
         for (int i = 0; i < 9; ++i) d[i] = F2(v0[i], v1[i]);
     }
-    if constexpr (FR) {
-        typename FrameStore<T>::type k0, k1;
-        const float s0 = frame_make<T>(c, m.dT.v.x, k0) - m.F.v.x;  // exact: frame values
-        const float s1 = frame_make<T>(c, m.dT.v.y, k1) - m.F.v.y;
-        const F2 sh(s0, s1);
-        h[0] = h[0] - c.wt0 * sh;
+    int8_t k0, k1;
+    const float s0 = frame_make(c, m.dT.v.x, k0) - m.F.v.x;  // exact: frame values
+    const float s1 = frame_make(c, m.dT.v.y, k1) - m.F.v.y;
+    const F2 sh(s0, s1);
+    h[0] = h[0] - c.wt0 * sh;
 #pragma unroll
-        for (int j = 1; j < 5; ++j) h[j] = h[j] - c.wt1 * sh;
-        if constexpr (VEC) {
-            if (in_plane(gm, off0, 2)) frame_st2<T>(at(dst.t, 0, off0), k0, k1);
-        } else {
-            if (in_plane(gm, off0)) dst.t[off0] = k0;
-            if (in_plane(gm, off1)) dst.t[off1] = k1;
-        }
+    for (int j = 1; j < 5; ++j) h[j] = h[j] - c.wt1 * sh;
+    if constexpr (VEC) {
+        if (in_plane(gm, off0, 2)) frame_st2<T>(at(dst.t, 0, off0), k0, k1);
+    } else {
+        if (in_plane(gm, off0)) dst.t[off0] = k0;
+        if (in_plane(gm, off1)) dst.t[off1] = k1;
     }
     if constexpr (VEC) {
         if (in_plane(gm, off0, 2)) {
@@ -640,13 +603,8 @@ __device__ __forceinline__ void collide_fluid_pair_x2(const Direct& c, const Geo
     }
     if constexpr (OBS) {
         // lane-wise IEEE sums: the same values as the scalar path
-        if constexpr (FR) {
-            obs_put(gm, obs, x0, y0, (double)m.F.v.x + (double)m.dTl.v.x);
-            obs_put(gm, obs, x1, y1, (double)m.F.v.y + (double)m.dTl.v.y);
-        } else {
-            obs_put(gm, obs, x0, y0, (double)m.dT.v.x);
-            obs_put(gm, obs, x1, y1, (double)m.dT.v.y);
-        }
+        obs_put(gm, obs, x0, y0, (double)m.F.v.x + (double)m.dTl.v.x);
+        obs_put(gm, obs, x1, y1, (double)m.F.v.y + (double)m.dTl.v.y);
     }
 }
 
@@ -658,11 +616,8 @@ __device__ __forceinline__ void update_fluid_pair_x2(const Direct& c, const Geom
     float a0[9], b0[5], a1[9], b1[5];
     pull<T>(src, gm, off0, a0, b0);
     pull<T>(src, gm, off1, a1, b1);
-    float F0 = 0.f, F1 = 0.f;
-    if constexpr (Framed<T>::value) {
-        F0 = frame_in<T>(c, src, gm, off0, b0);
-        F1 = frame_in<T>(c, src, gm, off1, b1);
-    }
+    const float F0 = frame_in<T>(c, src, gm, off0, b0);
+    const float F1 = frame_in<T>(c, src, gm, off1, b1);
     const Drag<float> r0 = drag_at<float, FIELD, typename T::P>(c, gm, phi, off0);
     const Drag<float> r1 = drag_at<float, FIELD, typename T::P>(c, gm, phi, off1);
     collide_fluid_pair_x2<T, OBS>(c, gm, dst, a0, b0, a1, b1, r0, r1, off0, off1, status, x0, y0, x1, y1, obs, F0,
@@ -803,14 +758,8 @@ __device__ __forceinline__ void update_pair(const CoefOf<T>& c, const Geom& gm, 
     using R = typename T::R;
     const bool f0 = v0 && x0 > 0 && x0 < gm.nx - 1 && y0 > 0 && y0 < gm.ny - 1;
     const bool f1 = v1 && x1 > 0 && x1 < gm.nx - 1 && y1 > 0 && y1 < gm.ny - 1;
-    if constexpr (Paired<T>::value) {
-        if (f0 && f1) {
-            update_fluid_pair_x2<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y0, x1, y1, status, obs);
-            return;
-        }
-    }
-    if constexpr (Core<T>::value) {
-        if (f0 && f1) {
+    if (f0 && f1) {
+        if constexpr (Core<T>::value) {
             R d0[9], h0[5], d1[9], h1[5];
             const int off0 = y0 * gm.pitch + x0, off1 = y1 * gm.pitch + x1;
             pull<T>(src, gm, off0, d0, h0);
@@ -819,8 +768,10 @@ __device__ __forceinline__ void update_pair(const CoefOf<T>& c, const Geom& gm, 
             const R F1 = core_frame_in<T>(c.k, src, gm, off1, h1);
             core_fluid_pair<T, FIELD, OBS, false>(c, gm, dst, phi, d0, h0, d1, h1, F0, F1, x0, y0, x1, y1, status,
                                                   obs);
-            return;
+        } else {
+            update_fluid_pair_x2<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y0, x1, y1, status, obs);
         }
+        return;
     }
     if (v0) update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x0, y0, status, obs);
     if (v1) update_node<T, FIELD, OBS>(c, gm, src, dst, phi, x1, y1, status, obs);
