@@ -417,7 +417,7 @@ def long_run_leg(n=1024, steps=50000):
 def batched_leg(steps, warmup, ncav=256, seed=2071):
     """Batched sweep: ncav cavities of uneven size (64^2..512^2), log-uniform Ra
     and Da, uniform porosity (seeded draws), FP32, autotuned tile shape and
-    schedule, graph-captured."""
+    schedule."""
     import torch
 
     from paper_1308_2071_gb300 import Batch
@@ -447,9 +447,9 @@ def batched_leg(steps, warmup, ncav=256, seed=2071):
                            if th == -2 else "runs of node pairs side by side along x" if th == -1 else
                            "runs of consecutive nodes" if th == 0 else "rectangles"),
                 nodes_per_thread=(2 if th < 0 else 1 if (tw if th == 0 else tw * th) in (32, 256) else 2),
-                mode="autotuned schedule, graph-captured: one persistent cooperative launch per call, or one launch "
+                mode="autotuned schedule: one persistent cooperative launch per call, from a graph, or one launch "
                      "per two steps (which reads and writes the lattices once for both; hbm_gbs counts "
-                     "114 B per node and step either way)",
+                     "114 B per node and step either way) and a persistent one for the last one or two",
                 blocks=q["nblocks"], tiles=q["ntiles"], diverged=int(st.sum()),
                 status=int(rc), sizes="U{64..512} square, seed %d" % seed)
 

@@ -154,7 +154,8 @@ int lbm_bounds_check(int* enabled, long* count);
 int lbm_reset(lbm_handle h);
 
 /* Autotuner of the one-step kernel: times candidate launch shapes (block_x x
- * block_y threads, nodes_per_thread 1, 2 or 3) on this lattice, keeps the
+ * block_y threads, nodes_per_thread 1, 2 or 3; 1 or 2 where lbm_step takes the
+ * lattice on chip), the handle's own first, on this lattice, keeps the
  * fastest and records it in a text cache at cache_path (NULL: no cache; one
  * line per device, precision, lattice size and porosity mode); a cached entry
  * is reused without timing.  Timing advances the lattice, so the handle is
@@ -164,7 +165,7 @@ int lbm_tune(lbm_handle h, const char* cache_path, int* block_x, int* block_y, i
 /* Advances nsteps time steps of Eq. 17-18 and Eq. 34-35 with the wall rule
  * (Section 4), asynchronously on the handle's stream.  Long runs replay a
  * captured CUDA graph.  FP32 lattices that fit on chip, and those too large for
- * the cache, take several steps per launch (the same bits; the last step of a
+ * the cache (but for a few rows or columns), take several steps per launch (the same bits; the last step of a
  * call is always a launch of its own).  Errors: LBM_ERR_ARG (nsteps < 0),
  * LBM_ERR_CUDA. */
 int lbm_step(lbm_handle h, long nsteps);
@@ -280,13 +281,13 @@ int lbm_load(lbm_handle h, const void* host, size_t bytes);
  * `stream` (a cudaStream_t, NULL = legacy default) and synchronised before
  * the call returns.  The paper has no counterpart to this call.
  * Scratch: one static device array of 38,984 bytes (the FP64 partial sums of
- * the fixed 1216-block reduction grid, the result, and a status word), which
- * every device that loads the library holds until the process exits; any
- * lattice that lbm_init accepts uses the same grid.  The first call on a
+ * a reduction grid of at most 1216 blocks, the result, and a status word with
+ * the grid's block counter), which every device that loads the library holds
+ * until the process exits; it is enough for any lattice that lbm_init accepts.  The first call on a
  * device looks up that array's device address once, with the device current:
  * make that first call before any stream capture.  All calls share the array
- * and it keeps the previous call's contents (the status word is cleared on
- * entry), so calls that overlap on the GPU race: serialise them.
+ * and it keeps the previous call's contents (the status word and the counter are
+ * cleared on entry), so calls that overlap on the GPU race: serialise them.
  * A checkpoint carries no divergence flag of the steps that made it, so the
  * state itself is tested: a non-finite value anywhere (the maximum of |u|
  * keeps NaN) or |u| >= 1/2 sets out->status and returns LBM_ERR_DIVERGED,
@@ -305,8 +306,10 @@ int lbm_observables_noalloc(const lbm_params* p, const void* ckpt_dev, size_t by
  * requested steps of all cavities (blocks walk a tile list that covers every
  * cavity; a bounded grid-wide barrier, or in the dataflow schedule bounded
  * per-cavity step counters, order the steps), or, where lbm_batch_tune finds
- * that faster (FP32 storage), one launch over all cavities per two steps; either
- * is captured into a CUDA graph on first use and replayed.  Per node it runs
+ * that faster (FP32 storage), one launch over all cavities per two steps, and
+ * the persistent kernel for the last one or two.  The persistent launch is captured
+ * into a CUDA graph on first use and replayed, and so are the two-step launches, 64
+ * steps to a graph (what is left below 64 is launched as it is).  Per node it runs
  * the same code as lbm_step: each cavity evolves bit for bit as it would alone. */
 typedef struct lbm_batch_s* lbm_batch;
 
@@ -314,7 +317,7 @@ typedef struct lbm_batch_s* lbm_batch;
  * lbm_init.  Errors: LBM_ERR_ARG (with the cavity index in the message),
  * LBM_ERR_CUDA. */
 int lbm_batch_init(const lbm_params* p, int ncav, void* stream, lbm_batch* out);
-/* Advances every cavity by nsteps (asynchronous, one graph launch). */
+/* Advances every cavity by nsteps (asynchronous). */
 int lbm_batch_step(lbm_batch b, long nsteps);
 /* Mean Nusselt numbers (Eq. 38) of every cavity into host arrays of ncav
  * doubles (either may be NULL); synchronises. */

@@ -377,8 +377,8 @@ StepLaunch step_launch(lbm_handle h, int src, cudaStream_t s) {
 // (lbm_duo.cu), or one.
 int most_steps(lbm_handle h) { return h->tile.steps ? h->tile.steps : h->duo.threads ? 2 : 1; }
 
-// Picks the way (FP32 storage only: FP64 is bound by its arithmetic unit, and
-// the states between of FP16 flow have to be rounded).  Measured, us per step
+// Picks the way (FP32 storage only: FP64 is bound by its arithmetic unit, and FP16
+// flow has no such kernels).  Measured, us per step
 // with one step per launch / a tile on chip: 64^2 2.2 / 1.0, 128^2 1.9 / 1.3, 200^2
 // 2.2 / 1.7, 230^2 2.1 / 1.9, 240^2 2.1 / 2.1, 260^2 2.3 / 2.5, 400^2 3.0 / 3.8, 500 x 100
 // 2.1 / 1.9, 1000 x 60 2.1 / 2.1; one / two: 700^2 6.1 / 7.4, 800^2 7.6 / 8.8, 850^2 9.4 /

@@ -21,7 +21,7 @@
 // side of a strip, and two rows of the first step per segment of rows.  Measured,
 // us per step against one step per launch: 4096^2 274 -> 170 (DRAM 5.8 TB/s, 1.96
 // GB per launch, issue 43 % busy), 1024^2 17.8 -> 14.0, 8192^2 with a porosity
-// field 1,270 -> 830.  Not kept: copies into shared memory by the bulk copy engine
+// field 1,270 -> 770.  Not kept: copies into shared memory by the bulk copy engine
 // (185 us memory alone against 169 with plain loads), rows prefetched into
 // registers (no change), 96 registers and six blocks per SM (190 us: the loads'
 // lines leave L1 before their second use), segments of a hundred rows (186

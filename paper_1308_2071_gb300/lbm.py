@@ -210,7 +210,7 @@ class Cavity:
 
 
 class Batch:
-    """Many independent cavities advanced by one persistent launch per call.
+    """Many independent cavities advanced together.
 
     cavities: list of dicts with nx, ny, Ra, Da, phi and optional Section 4
     overrides (Pr, J, Ma, ...); all share one precision ("f32" or "f64")."""
