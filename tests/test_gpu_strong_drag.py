@@ -67,3 +67,18 @@ def test_the_drag_stays_at_its_bound(precision, solid):
     obs = c.observables(check=False)
     c.close()
     assert obs["status"] == 0 and 0.0 <= obs["umax"] < 1e-30
+
+
+@pytest.mark.parametrize("least", [1e-8, 1e-6, 1e-4])
+@pytest.mark.parametrize("precision", ["f32", "f32t"])
+def test_max_speed_where_a_small_porosity_varies(precision, least):
+    # by 5 % a row: v near the walls is 1e10 .. 1e2 times u.  Against the FP64 run; FP32's 21
+    # steps and its drag (see above) take some hundred roundings of 6e-8, far below 1 %
+    phi = np.geomspace(least, 4.8 * least, 30 * 37).reshape(30, 37)
+    umax = {}
+    for prec in ("f64", precision):
+        c = cavity(prec, phi)
+        c.step(21)
+        umax[prec] = c.observables(check=False)["umax"]
+        c.close()
+    assert abs(umax[precision] - umax["f64"]) <= 1e-2 * umax["f64"]
