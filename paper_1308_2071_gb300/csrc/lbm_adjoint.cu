@@ -161,8 +161,8 @@ struct Divider {
 // 10.8 ms instead of 10.0 for the call below).
 //
 // Everything but the forward states stays in L2; a step moves 72 MB through it
-// at 512^2 and is bound by that latency and by issue slots (540 instructions per
-// pair, 202 of them arithmetic; 1.35 waves of 20 warps per SM).  512^2 FP32, us
+// at 512^2 and is bound by that latency and by issue slots (545 instructions per
+// pair, some 205 of them arithmetic; 1.35 waves of 20 warps per SM).  512^2 FP32, us
 // per reverse step alone: 7.6; 8.3 with an index per access, and 23.4 for the
 // direct formulas in one kernel for the interior and one for the ring of nodes
 // near the walls on a stream of its own.  The gradient of 600 steps: 19.8 -> 9.8 ms.
